@@ -213,9 +213,8 @@ extern "C" rr_status rr_batch_create(const rr_wavefront *fronts, uint32_t n_fron
     std::vector<BatchScene> segs(n_fronts);
     for (uint32_t k = 0; k < n_fronts; ++k) {
         const rr_bvh *h = fronts[k].bvh;
-        segs[k].nodes = reinterpret_cast<const float4 *>(h->nodes);
-        segs[k].tris = reinterpret_cast<const float4 *>(h->tris);
-        segs[k].planes = h->planes;
+        segs[k].nodes = h->nodes;
+        segs[k].tris = h->tris;
         segs[k].n_nodes = h->n_nodes;
         segs[k].n_tris = h->n_tris;
         segs[k].table = accumulating(b) ? fronts[k].table->cells : nullptr;

@@ -12,9 +12,8 @@ constexpr uint32_t kMaxBatchSegments = 1024;
 // Device descriptor of one wavefront (segment) of a batch: its scene's BVH,
 // the quantisation frame of its box, and its length table (or null).
 struct BatchScene {
-    const float4 *nodes;
-    const float4 *tris;
-    const float4 *planes;
+    const DevNode *nodes;
+    const DevTri *tris;
     uint32_t n_nodes;
     uint32_t n_tris;
     unsigned long long *table;  // cells {sum, count}; null: no adaptive estimate, no update

@@ -9,6 +9,7 @@
 #include <mutex>
 #include <string>
 #include <unordered_map>
+#include <vector>
 
 #include "../../include/rr.h"
 
@@ -172,11 +173,41 @@ struct alignas(16) RRTri {
     float4 e2;
 };
 
+// The forms the trace kernel reads, built from the two above at upload.  Each
+// is a whole number of 32-byte sectors, so a node takes three and a triangle
+// two 256-bit loads: with divergent lanes every load of a lane is a wavefront
+// of its own in the L1 data pipe, whatever its width, and that pipe is what
+// incoherent rays fill first (80-byte nodes by five and 48-byte triangles by
+// three 128-bit loads kept it 68% busy on two million random-order rays).
+//   masks: imask | valid << 8.  q: low and high planes per axis, x y z.
+struct alignas(32) DevNode {
+    float px, py, pz;
+    uint32_t masks;
+    float sx, sy, sz;  // the steps 2^(e - 127)
+    uint32_t child_base;
+    uint8_t qlo_x[8], qhi_x[8], qlo_y[8], qhi_y[8];
+    uint8_t qlo_z[8], qhi_z[8];
+    uint32_t tri_base;
+    uint32_t tribits;
+    uint32_t unused[2];
+};
+static_assert(sizeof(DevNode) == 96, "device node layout");
+
+// v0, e1, e2, the original id, and the normal (v1-v0)x(v2-v0) as hi + lo floats.
+struct alignas(32) DevTri {
+    float v0[3], e1[3], e2[3];
+    uint32_t id;
+    float nhi[3], nlo[3];
+};
+static_assert(sizeof(DevTri) == 64, "device triangle layout");
+
 struct rr_bvh {
     int device;
-    RRNode8 *nodes;   // device
-    RRTri *tris;      // device
-    float4 *planes;   // device, two per triangle (normal as hi + lo floats)
+    DevNode *nodes;   // device
+    DevTri *tris;     // device, in BVH order
+    // the padding words of a deserialized buffer's triangles and planes (four
+    // per triangle), kept only when some are not zero: serializing returns them
+    std::vector<float> padding;
     uint32_t n_nodes;
     uint32_t n_tris;
     uint32_t root_is_leaf;  // scenes of 1..4 triangles: no inner node, the root is one leaf

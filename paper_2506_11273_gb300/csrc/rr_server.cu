@@ -434,9 +434,8 @@ extern "C" rr_status rr_server_add_scene(rr_server *s, const rr_bvh *bvh, rr_len
     }
     // the descriptor, with the quantisation frame computed on the device
     BatchScene h{};
-    h.nodes = reinterpret_cast<const float4 *>(bvh->nodes);
-    h.tris = reinterpret_cast<const float4 *>(bvh->tris);
-    h.planes = bvh->planes;
+    h.nodes = bvh->nodes;
+    h.tris = bvh->tris;
     h.n_nodes = bvh->n_nodes;
     h.n_tris = bvh->n_tris;
     h.table = adaptive(s) ? table->cells : nullptr;

@@ -6,9 +6,22 @@
 // effect on control-flow and cache efficiency).  Each thread walks the
 // compressed 8-wide BVH with a stack of node groups (the hit children of a
 // node that remain to be visited, in the near-to-far order given by the ray's
-// direction octant); the leaves a node's children hit are tested at once.
-// Triangles are intersected with Moller-Trumbore in fp32 and the winning
-// distance is refined in compensated fp32.
+// direction octant).  Triangles are intersected with Moller-Trumbore in fp32
+// and the winning distance is refined in compensated fp32.
+//
+// What bounds it: instruction issue for coherent rays, the L1 data pipe and L2
+// latency for incoherent ones, and for small launches the latency of the
+// longest ray.  A step of the loop therefore serves both kinds of work: a lane
+// tests one pending triangle and visits one node, with room for two pending
+// triangle groups, so that 25 of 32 lanes are in the node branch (20 when a
+// step was either a triangle or a node; a simulation of the exact traversal on
+// 150,000 random-order rays).  Nodes and triangles are read by 256-bit loads,
+// two slots share a packed multiply-add, the top of the stack is in shared
+// memory, and a warp whose last rays run on hands each to four lanes.
+// Measured against the earlier form (one step a triangle or a node, 128-bit
+// loads of 80-byte nodes, local stack), 1,168,576 triangles: 2.07M camera rays
+// 0.723 -> 0.582 ms, 8.3M random-order secondary rays 3.38 -> 2.78 ms, 0.99M
+// any-hit shadow rays 0.273 -> 0.235 ms.
 //
 // Two variants serve the reordering study: indirect access (the queue hands
 // out positions of an index buffer, so sorted rays are traced without being
@@ -16,6 +29,7 @@
 // triangle found inside the interval ends the ray, Section 4).
 #include <chrono>
 #include <cmath>
+#include <cstring>
 
 #include "rr_batch.cuh"
 #include "rr_common.cuh"
@@ -28,9 +42,8 @@ constexpr int kTraceBlock = 128;
 
 // The BVH arrays of one scene.
 struct SceneRef {
-    const float4 *nodes;   // RRNode8 as five float4
-    const float4 *tris;    // RRTri as three float4
-    const float4 *planes;  // two float4 per triangle: normal hi.xyz, lo.x | lo.y, lo.z
+    const DevNode *nodes;
+    const DevTri *tris;
     uint32_t n_nodes;
     uint32_t n_tris;
 };
@@ -52,9 +65,29 @@ struct TraceArgs {
     uint32_t n_segs;
 };
 
+// Reciprocal of a direction component, kept finite: the hardware estimate (1
+// ulp) and one Newton step in fused arithmetic, which rounds 1/m correctly
+// unless m's mantissa is all ones (Markstein, IBM J. Res. Dev. 34(1), 1990).
+// The rounded intrinsic gives the same box tests; its range checks, at the few
+// lanes of a refill, cost 3% of a camera-ray trace.
 __device__ __forceinline__ float safe_inv(float x) {
     const float m = fabsf(x) > 1e-18f ? x : copysignf(1e-18f, x);
-    return __frcp_rn(m);
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(m));
+    const float z = fmaf(y, fmaf(-m, y, 1.0f), y);
+    return y == 0.0f ? y : z;  // an infinite m
+}
+
+// Eight 32-bit words by one 256-bit load (32-byte aligned, read-only data).
+struct Words8 {
+    uint32_t w[8];
+};
+__device__ __forceinline__ Words8 load256(const void *p) {
+    Words8 r;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7])
+        : "l"(p));
+    return r;
 }
 
 // Error-free transformations (Knuth's TwoSum, FMA-based TwoProd).
@@ -73,11 +106,12 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
 // stored as hi + lo floats and v0 - o split exactly into hi + lo.  Plain fp32
 // loses relative accuracy when the hit is close to the origin compared with
 // |v0 - o|; this form keeps it at a few ulps.
-__device__ __forceinline__ float refine_t(const SceneRef &a, uint32_t k, float4 o, float4 d) {
-    const float4 v0 = __ldg(a.tris + 3 * (size_t)k);
-    const float4 p0 = __ldg(a.planes + 2 * (size_t)k), p1 = __ldg(a.planes + 2 * (size_t)k + 1);
-    const float nh[3] = {p0.x, p0.y, p0.z}, nl[3] = {p0.w, p1.x, p1.y};
-    const float vo[3] = {v0.x, v0.y, v0.z}, oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z};
+__device__ __forceinline__ float refine_t(const SceneRef &a, uint32_t k, float4 o, float3 d) {
+    const DevTri *tp = a.tris + k;
+    const float nh[3] = {__ldg(tp->nhi), __ldg(tp->nhi + 1), __ldg(tp->nhi + 2)};
+    const float nl[3] = {__ldg(tp->nlo), __ldg(tp->nlo + 1), __ldg(tp->nlo + 2)};
+    const float vo[3] = {__ldg(tp->v0), __ldg(tp->v0 + 1), __ldg(tp->v0 + 2)};
+    const float oo[3] = {o.x, o.y, o.z}, dd[3] = {d.x, d.y, d.z};
     float num_hi = 0.0f, num_lo = 0.0f, den_hi = 0.0f, den_lo = 0.0f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -102,44 +136,186 @@ __device__ __forceinline__ float byte_plus_2p23(uint32_t w) {
     return __uint_as_float(__byte_perm(w, 0x4B000000u, (uint32_t)K | 0x7540u));
 }
 
-// Traversal state of the ray a lane is tracing.  Node groups (child base,
-// remaining hit mask in the near-to-far order of the ray's direction octant,
-// inner-child mask) are the stack entries: one push per level descended.
+// The hit children of a node, as octant-ordered inner children, and the
+// triangles of its hit leaves.  Triangle groups wait in a first-in first-out
+// queue, so triangles are always tested in the order in which the traversal
+// met them.
+struct TriGroup {
+    uint32_t base;  // the node's first triangle
+    uint32_t hits;  // triangle bits still to test
+    uint32_t all;   // the node's triangle bits (a bit's rank among them numbers its triangle)
+};
+
+// Traversal state of a ray.  Node groups (child base, remaining hit mask in
+// the near-to-far order of the ray's direction octant | inner-child mask << 8)
+// are the stack entries: one push per level descended.
 struct RayState {
-    float4 o, d;
+    float4 o;  // origin, tmin
     float idx, idy, idz;
     uint32_t negmask;
-    float best, bu, bv;
-    uint32_t best_tri, best_k;
-    uint32_t g_base, g_hits, g_imask;
-    uint32_t t_base, t_hits, t_all;  // pending triangle group: base, bits to test, node's tribits
+    float best;               // distance of the nearest triangle so far, or tmax
+    uint32_t g_base, g_mask;  // current node group
+    TriGroup t;               // the triangle group being tested
+    uint32_t u_hits;          // the triangle bits of the group after it (0: none)
     int sp;
 };
 
-__device__ __forceinline__ void ray_begin(RayState &r, const SceneRef &a, float4 o, float4 d) {
+// The nearest triangle so far: barycentrics and BVH-ordered number (kMiss
+// before the first hit).
+struct Hit {
+    float u, v;
+    uint32_t k;
+};
+
+// Stack entries a lane keeps in shared memory; deeper ones go to local memory.
+// An incoherent ray's local stack misses L1 on half of its pops, in front of
+// the node load that needs the entry.
+constexpr int kSharedStack = 8;
+
+// What the node visits do not need, besides RayState: the direction (read by
+// triangle tests), the hit record (written about once per ray), and base and
+// bits of the second triangle group.  Three ways to keep it:
+//  - one scene: the hit record in shared memory, the rest in registers: 64
+//    registers a thread without spills, 32 warps per SM;
+//  - several scenes in 128-thread blocks (LEAN): all of it in shared memory: 56 registers, 36 warps per SM,
+//    and 1,024 registers of the SM stay free, so that the one-warp blocks of the
+//    host-link copy kernel run beside a full trace;
+//  - four lanes to a ray: in registers (RegisterExtra).
+// The other way round each was slower: one scene at 56 registers 2.91 against
+// 2.77 ms for 8.3M random-order rays and 0.602 against 0.581 ms for 2.07M camera
+// rays; several scenes at 64 registers 1.244 against 1.231 ms for the 3.7M rays
+// of a batch of twelve wavefronts.
+template <bool MULTI, int BLOCK>
+constexpr bool trace_lean() {
+    return MULTI && BLOCK == 128;
+}
+template <bool LEAN, int BLOCK>
+struct LaneMem {
+    float4 hit[BLOCK];
+    uint2 stack[kSharedStack * BLOCK];
+    float4 d[LEAN ? BLOCK : 1];
+    uint2 u[LEAN ? BLOCK : 1];
+};
+template <bool LEAN, int BLOCK>
+struct LaneExtra {
+    LaneMem<LEAN, BLOCK> &m;
+    uint32_t at;  // thread of the block
+    float3 dir;   // unless LEAN
+    uint2 second;
+    __device__ __forceinline__ void begin(float4 d) {
+        if (LEAN)
+            m.d[at] = d;
+        else
+            dir = make_float3(d.x, d.y, d.z);
+        set_hit(0.0f, 0.0f, kMiss);
+    }
+    __device__ __forceinline__ float3 d() const {
+        if (!LEAN) return dir;
+        const float4 x = m.d[at];
+        return make_float3(x.x, x.y, x.z);
+    }
+    __device__ __forceinline__ void set_hit(float u, float v, uint32_t k) {
+        m.hit[at] = make_float4(u, v, __uint_as_float(k), 0.0f);
+    }
+    __device__ __forceinline__ Hit hit() const {
+        const float4 h = m.hit[at];
+        return Hit{h.x, h.y, __float_as_uint(h.z)};
+    }
+    __device__ __forceinline__ void set_u(uint32_t base, uint32_t all) {
+        if (LEAN)
+            m.u[at] = make_uint2(base, all);
+        else
+            second = make_uint2(base, all);
+    }
+    __device__ __forceinline__ uint2 u() const { return LEAN ? m.u[at] : second; }
+};
+// The same in registers, where four lanes share a ray.
+struct RegisterExtra {
+    float3 dir;
+    Hit best;
+    uint2 second;
+    __device__ __forceinline__ void begin(float4 d) {
+        dir = make_float3(d.x, d.y, d.z);
+        best = Hit{0.0f, 0.0f, kMiss};
+        second = make_uint2(0u, 0u);
+    }
+    __device__ __forceinline__ float3 d() const { return dir; }
+    __device__ __forceinline__ void set_hit(float u, float v, uint32_t k) { best = Hit{u, v, k}; }
+    __device__ __forceinline__ Hit hit() const { return best; }
+    __device__ __forceinline__ void set_u(uint32_t base, uint32_t all) { second = make_uint2(base, all); }
+    __device__ __forceinline__ uint2 u() const { return second; }
+};
+
+// Drops everything the ray still had to visit.
+__device__ __forceinline__ void ray_stop(RayState &r) {
+    r.g_mask = 0u;
+    r.t.hits = 0u;
+    r.u_hits = 0u;
+    r.sp = 0;
+}
+
+// The second triangle group moves up once the first is tested.
+template <typename X>
+__device__ __forceinline__ void next_group(RayState &r, const X &x) {
+    if (r.t.hits == 0u && r.u_hits != 0u) {
+        const uint2 u = x.u();
+        r.t.base = u.x;
+        r.t.hits = r.u_hits;
+        r.t.all = u.y;
+        r.u_hits = 0u;
+    }
+}
+
+template <typename X>
+__device__ __forceinline__ void ray_begin(RayState &r, X &x, const SceneRef &a, float4 o, float4 d) {
+    x.begin(d);
     r.o = o;
-    r.d = d;
     r.idx = safe_inv(d.x);
     r.idy = safe_inv(d.y);
     r.idz = safe_inv(d.z);
     r.negmask = (r.idx < 0.0f ? 1u : 0u) | (r.idy < 0.0f ? 2u : 0u) | (r.idz < 0.0f ? 4u : 0u);
     r.best = d.w;
-    r.bu = 0.0f;
-    r.bv = 0.0f;
-    r.best_tri = kMiss;
-    r.best_k = 0u;
     // the current node group starts as a virtual group holding only the root
     r.g_base = 0u;
-    r.g_hits = (a.n_nodes > 0 && o.w <= d.w) ? 1u : 0u;
-    r.g_imask = 1u << r.negmask;
-    r.t_base = 0u;
-    r.t_hits = 0u;
-    r.t_all = 0u;
+    r.g_mask = ((a.n_nodes > 0 && o.w <= d.w) ? 1u : 0u) | (0x100u << r.negmask);
+    r.t.base = r.t.hits = r.t.all = 0u;
+    r.u_hits = 0u;
     r.sp = 0;
 }
 
-// Stack entries are node groups: (child base, remaining hit mask in octant
-// order | inner-child mask << 8).
+// Takes the nearest child of the current node group (which holds one); what
+// remains of the group is left in r.g_mask.
+__device__ __forceinline__ uint32_t take_child(RayState &r) {
+    const uint32_t pos = __ffs(r.g_mask) - 1u;
+    r.g_mask &= r.g_mask - 1u;
+    const uint32_t slot = pos ^ r.negmask;
+    return r.g_base + __popc((r.g_mask >> 8) & ((1u << slot) - 1u));
+}
+
+// Hit masks of slot bits to octant positions (bit s to bit s ^ octant), a
+// table in shared memory: the three conditional swaps it replaces are a tenth
+// of the node visit's ALU work.
+struct OctantTable {
+    alignas(16) uint8_t at[8 * 256];
+};
+constexpr OctantTable octant_table() {
+    OctantTable t{};
+    for (uint32_t k = 0; k < 8 * 256; ++k) {
+        uint32_t h = k & 255u;
+        if (k & 256u) h = ((h & 0x55u) << 1) | ((h >> 1) & 0x55u);
+        if (k & 512u) h = ((h & 0x33u) << 2) | ((h >> 2) & 0x33u);
+        if (k & 1024u) h = ((h & 0x0Fu) << 4) | (h >> 4);
+        t.at[k] = (uint8_t)h;
+    }
+    return t;
+}
+__device__ const OctantTable g_octant_table = octant_table();
+__device__ __forceinline__ const uint8_t *block_octant_table() {
+    __shared__ OctantTable s_oct;
+    for (uint32_t k = threadIdx.x; k < 128u; k += blockDim.x)
+        reinterpret_cast<uint4 *>(s_oct.at)[k] = reinterpret_cast<const uint4 *>(g_octant_table.at)[k];
+    return s_oct.at;
+}
 
 __device__ __forceinline__ float max3f(float a, float b, float c) {
     float r;
@@ -152,150 +328,162 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
     return r;
 }
 
-// Node part of a traversal round: visit the nearest node of the current group
-// (its hit inner children become the current group, its hit leaves the
-// pending triangle group).
-__device__ __forceinline__ bool ray_visit_node(RayState &r, uint2 *stack, const SceneRef &a, uint32_t *err) {
-    const float tmin = r.o.w;
-    const uint32_t pos = __ffs(r.g_hits) - 1u;
-    r.g_hits &= r.g_hits - 1u;
-    const uint32_t slot = pos ^ r.negmask;
-    const uint32_t node = r.g_base + __popc(r.g_imask & ((1u << slot) - 1u));
-    if (!index_ok(node, a.n_nodes, err)) {  // checked build: end the ray as a miss
-        r.best_tri = kMiss;
-        r.g_hits = 0u;
-        r.t_hits = 0u;
-        r.sp = 0;
-        return true;
-    }
-    if (r.g_hits != 0u) {
-        if (r.sp >= (int)kTraceStack) return false;
-        stack[r.sp++] = make_uint2(r.g_base, r.g_hits | (r.g_imask << 8));
-    }
-    const float4 *np = a.nodes + 5 * (size_t)node;
-    const float4 f0 = __ldg(np), f1 = __ldg(np + 1), f2 = __ldg(np + 2), f3 = __ldg(np + 3), f4 = __ldg(np + 4);
-    const uint32_t ew = __float_as_uint(f0.w);
-    const float sx = __uint_as_float((ew & 0xFFu) << 23);
-    const float sy = __uint_as_float(((ew >> 8) & 0xFFu) << 23);
-    const float sz = __uint_as_float(((ew >> 16) & 0xFFu) << 23);
-    // plane of quantised value q: t = q*b + a.  The byte arrives as 2^23 + q, so
-    // the offset moves into a: a' = a - 2^23*b.  Rounding a' costs at most half
-    // a quantisation step, and every stored box is one step larger than the
-    // child it bounds.
-    const float bx = sx * r.idx, by = sy * r.idy, bz = sz * r.idz;
-    const float ax = fmaf(-8388608.0f, bx, (f0.x - r.o.x) * r.idx);
-    const float ay = fmaf(-8388608.0f, by, (f0.y - r.o.y) * r.idy);
-    const float az = fmaf(-8388608.0f, bz, (f0.z - r.o.z) * r.idz);
-    uint32_t nxl = __float_as_uint(f2.x), nxh = __float_as_uint(f2.y);
-    uint32_t nyl = __float_as_uint(f2.z), nyh = __float_as_uint(f2.w);
-    uint32_t nzl = __float_as_uint(f3.x), nzh = __float_as_uint(f3.y);
-    uint32_t fxl = __float_as_uint(f3.z), fxh = __float_as_uint(f3.w);
-    uint32_t fyl = __float_as_uint(f4.x), fyh = __float_as_uint(f4.y);
-    uint32_t fzl = __float_as_uint(f4.z), fzh = __float_as_uint(f4.w);
-    // for a negative direction the near plane is the box's high side
-    if (r.negmask & 1u) {
-        const uint32_t t0 = nxl, t1 = nxh;
-        nxl = fxl; nxh = fxh; fxl = t0; fxh = t1;
-    }
-    if (r.negmask & 2u) {
-        const uint32_t t0 = nyl, t1 = nyh;
-        nyl = fyl; nyh = fyh; fyl = t0; fyh = t1;
-    }
-    if (r.negmask & 4u) {
-        const uint32_t t0 = nzl, t1 = nzh;
-        nzl = fzl; nzh = fzh; fzl = t0; fzh = t1;
-    }
-    uint32_t hm = 0u;  // slot s: the ray meets the child's box within [tmin, best]
-    const float best = r.best;
-#define RR_SLOT(S)                                                                                      \
-    {                                                                                                   \
-        const uint32_t w_nx = (S) < 4 ? nxl : nxh, w_ny = (S) < 4 ? nyl : nyh, w_nz = (S) < 4 ? nzl : nzh; \
-        const uint32_t w_fx = (S) < 4 ? fxl : fxh, w_fy = (S) < 4 ? fyl : fyh, w_fz = (S) < 4 ? fzl : fzh; \
-        const float t0 = max3f(fmaf(byte_plus_2p23<(S) & 3>(w_nx), bx, ax),                              \
-                               fmaf(byte_plus_2p23<(S) & 3>(w_ny), by, ay),                              \
-                               fmaxf(fmaf(byte_plus_2p23<(S) & 3>(w_nz), bz, az), tmin));                \
-        const float t1 = min3f(fmaf(byte_plus_2p23<(S) & 3>(w_fx), bx, ax),                              \
-                               fmaf(byte_plus_2p23<(S) & 3>(w_fy), by, ay),                              \
-                               fminf(fmaf(byte_plus_2p23<(S) & 3>(w_fz), bz, az), best));                \
-        if (t0 <= t1) hm |= 1u << (S);                                                                  \
-    }
-    RR_SLOT(0) RR_SLOT(1) RR_SLOT(2) RR_SLOT(3) RR_SLOT(4) RR_SLOT(5) RR_SLOT(6) RR_SLOT(7)
-#undef RR_SLOT
-    const uint32_t imask = (ew >> 24) & 0xFFu, tribits = __float_as_uint(f1.z);
-    hm &= __float_as_uint(f1.w);  // used slots only
-    // inner children to octant positions: bit s -> bit s ^ negmask
-    uint32_t hits = hm & imask;
-    if (r.negmask & 1u) hits = ((hits & 0x55u) << 1) | ((hits >> 1) & 0x55u);
-    if (r.negmask & 2u) hits = ((hits & 0x33u) << 2) | ((hits >> 2) & 0x33u);
-    if (r.negmask & 4u) hits = ((hits & 0x0Fu) << 4) | (hits >> 4);
-    // leaves: slot bit s -> nibble s, keeping the triangles the nibble holds
-    uint32_t x = hm & ~imask;
-    x = (x | (x << 12)) & 0x000F000Fu;
-    x = (x | (x << 6)) & 0x03030303u;
-    x = (x | (x << 3)) & 0x11111111u;
-    const uint32_t tris = (x * 15u) & tribits;
-    r.g_base = __float_as_uint(f1.x);
-    r.g_hits = hits;
-    r.g_imask = imask;
-    r.t_base = __float_as_uint(f1.y);
-    r.t_hits = tris;
-    r.t_all = tribits;
-    return true;
+// Two fused multiply-adds in one instruction, each rounded as fmaf.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 r;
+    asm("{\n"
+        "  .reg .b64 x, y, z, w;\n"
+        "  mov.b64 x, {%2, %3};\n"
+        "  mov.b64 y, {%4, %5};\n"
+        "  mov.b64 z, {%6, %7};\n"
+        "  fma.rn.f32x2 w, x, y, z;\n"
+        "  mov.b64 {%0, %1}, w;\n"
+        "}\n"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
 }
 
-// Tests the nearest-slot triangle of the pending group (one triangle per
-// traversal step).  ANY: a hit ends the ray (the pending group, the current
-// node group and the stack are dropped).
-template <bool ANY>
-__device__ __forceinline__ void test_one_triangle(RayState &r, const SceneRef &a, uint32_t *err) {
-    const float tmin = r.o.w;
-    const uint32_t b = __ffs(r.t_hits) - 1u;
-    r.t_hits &= r.t_hits - 1u;
-    const uint32_t k = r.t_base + __popc(r.t_all & ((1u << b) - 1u));
-    if (!index_ok(k, a.n_tris, err)) return;
-    const float4 *tp = a.tris + 3 * (size_t)k;
-    const float4 v0 = __ldg(tp), e1 = __ldg(tp + 1), e2 = __ldg(tp + 2);
-    const float4 d = r.d, o = r.o;
-    const float pvx = d.y * e2.z - d.z * e2.y;
-    const float pvy = d.z * e2.x - d.x * e2.z;
-    const float pvz = d.x * e2.y - d.y * e2.x;
-    const float det = e1.x * pvx + e1.y * pvy + e1.z * pvz;
-    if (det == 0.0f) return;
-    const float inv = __frcp_rn(det);
-    const float tvx = o.x - v0.x, tvy = o.y - v0.y, tvz = o.z - v0.z;
-    const float u = (tvx * pvx + tvy * pvy + tvz * pvz) * inv;
-    if (!(u >= 0.0f && u <= 1.0f)) return;
-    const float qvx = tvy * e1.z - tvz * e1.y;
-    const float qvy = tvz * e1.x - tvx * e1.z;
-    const float qvz = tvx * e1.y - tvy * e1.x;
-    const float v = (d.x * qvx + d.y * qvy + d.z * qvz) * inv;
-    if (!(v >= 0.0f && u + v <= 1.0f)) return;
-    const float t = (e2.x * qvx + e2.y * qvy + e2.z * qvz) * inv;
-    if (t > tmin && t < r.best) {
-        r.best = t;
-        r.bu = u;
-        r.bv = v;
-        r.best_tri = __float_as_uint(v0.w);
-        r.best_k = k;
-        if (ANY) {
-            r.t_hits = 0u;
-            r.g_hits = 0u;
-            r.sp = 0;
+// A node's slabs along a ray: plane q of an axis lies at t = q*b + a.  The
+// byte arrives as 2^23 + q, so the offset moves into a: a' = a - 2^23*b.
+// Rounding a' costs at most half a quantisation step, and every stored box is
+// one step larger than the child it bounds.  n, f: near and far planes per
+// axis, slots 0..3 and 4..7.
+struct NodeSlabs {
+    float ax, ay, az, bx, by, bz;
+    uint32_t nx[2], ny[2], nz[2], fx[2], fy[2], fz[2];
+};
+__device__ __forceinline__ NodeSlabs node_slabs(const RayState &r, const Words8 &n0, const Words8 &n1,
+                                                const Words8 &n2) {
+    NodeSlabs s;
+    s.bx = __uint_as_float(n0.w[4]) * r.idx;
+    s.by = __uint_as_float(n0.w[5]) * r.idy;
+    s.bz = __uint_as_float(n0.w[6]) * r.idz;
+    s.ax = fmaf(-8388608.0f, s.bx, (__uint_as_float(n0.w[0]) - r.o.x) * r.idx);
+    s.ay = fmaf(-8388608.0f, s.by, (__uint_as_float(n0.w[1]) - r.o.y) * r.idy);
+    s.az = fmaf(-8388608.0f, s.bz, (__uint_as_float(n0.w[2]) - r.o.z) * r.idz);
+    // for a negative direction the near plane is the box's high side
+    const bool sx = r.negmask & 1u, sy = r.negmask & 2u, sz = r.negmask & 4u;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        s.nx[h] = sx ? n1.w[2 + h] : n1.w[h];
+        s.fx[h] = sx ? n1.w[h] : n1.w[2 + h];
+        s.ny[h] = sy ? n1.w[6 + h] : n1.w[4 + h];
+        s.fy[h] = sy ? n1.w[4 + h] : n1.w[6 + h];
+        s.nz[h] = sz ? n2.w[2 + h] : n2.w[h];
+        s.fz[h] = sz ? n2.w[h] : n2.w[2 + h];
+    }
+    return s;
+}
+
+// The hit slots of a visited node become the ray's current group (inner
+// children) and its last pending triangle group (leaves).
+template <typename X>
+__device__ __forceinline__ void take_hits(RayState &r, X &x, const Words8 &n0, const Words8 &n2, uint32_t hm,
+                                          const uint8_t *s_oct) {
+    const uint32_t imask = n0.w[3] & 0xFFu, tribits = n2.w[5];
+    hm &= n0.w[3] >> 8;  // used slots only
+    const uint32_t hits = s_oct[r.negmask * 256u + (hm & imask)];
+    // leaves: slot bit s -> nibble s, keeping the triangles the nibble holds
+    uint32_t leaf = hm & ~imask;
+    leaf = (leaf | (leaf << 12)) & 0x000F000Fu;
+    leaf = (leaf | (leaf << 6)) & 0x03030303u;
+    leaf = (leaf | (leaf << 3)) & 0x11111111u;
+    const uint32_t tris = (leaf * 15u) & tribits;
+    r.g_base = n0.w[7];
+    r.g_mask = hits | (imask << 8);
+    if (tris != 0u) {
+        if (r.t.hits == 0u) {
+            r.t.base = n2.w[4];
+            r.t.hits = tris;
+            r.t.all = tribits;
+        } else {
+            x.set_u(n2.w[4], tribits);
+            r.u_hits = tris;
         }
     }
 }
 
-__device__ __forceinline__ float4 ray_result(const RayState &r, const SceneRef &a) {
-    if (r.best_tri == kMiss) return make_float4(__int_as_float(0x7f800000), 0.0f, 0.0f, __uint_as_float(kMiss));
-    const float tr = refine_t(a, r.best_k, r.o, r.d);
-    return make_float4(isfinite(tr) ? tr : r.best, r.bu, r.bv, __uint_as_float(r.best_tri));
+// The slots of a node whose box the ray meets within [tmin, best], two slots
+// to a fused multiply-add instruction.
+__device__ __forceinline__ uint32_t hit_slots(const RayState &r, const NodeSlabs &s) {
+    const float tmin = r.o.w, best = r.best;
+    const float2 bx = make_float2(s.bx, s.bx), by = make_float2(s.by, s.by), bz = make_float2(s.bz, s.bz);
+    const float2 ax = make_float2(s.ax, s.ax), ay = make_float2(s.ay, s.ay), az = make_float2(s.az, s.az);
+    uint32_t hm = 0u;
+#define RR_BYTES(S, W) make_float2(byte_plus_2p23<(S) & 3>(W[(S) / 4]), byte_plus_2p23<((S) & 3) + 1>(W[(S) / 4]))
+#define RR_SLOTS(S)                                                                                          \
+    {                                                                                                        \
+        const float2 nx = fma2(RR_BYTES(S, s.nx), bx, ax), fx = fma2(RR_BYTES(S, s.fx), bx, ax);              \
+        const float2 ny = fma2(RR_BYTES(S, s.ny), by, ay), fy = fma2(RR_BYTES(S, s.fy), by, ay);              \
+        const float2 nz = fma2(RR_BYTES(S, s.nz), bz, az), fz = fma2(RR_BYTES(S, s.fz), bz, az);              \
+        if (max3f(nx.x, ny.x, fmaxf(nz.x, tmin)) <= min3f(fx.x, fy.x, fminf(fz.x, best))) hm |= 1u << (S);    \
+        if (max3f(nx.y, ny.y, fmaxf(nz.y, tmin)) <= min3f(fx.y, fy.y, fminf(fz.y, best))) hm |= 2u << (S);    \
+    }
+    RR_SLOTS(0) RR_SLOTS(2) RR_SLOTS(4) RR_SLOTS(6)
+#undef RR_SLOTS
+#undef RR_BYTES
+    return hm;
+}
+
+// Moller-Trumbore of triangle k: true (with u, v, t) for a hit with
+// tmin < t < best.
+__device__ __forceinline__ bool meet_triangle(const RayState &r, float3 d, const SceneRef &a, uint32_t k, float &u,
+                                              float &v, float &t) {
+    const DevTri *tp = a.tris + k;
+    const Words8 w = load256(tp);
+    const float3 v0 = make_float3(__uint_as_float(w.w[0]), __uint_as_float(w.w[1]), __uint_as_float(w.w[2]));
+    const float3 e1 = make_float3(__uint_as_float(w.w[3]), __uint_as_float(w.w[4]), __uint_as_float(w.w[5]));
+    const float3 e2 = make_float3(__uint_as_float(w.w[6]), __uint_as_float(w.w[7]), __ldg(&tp->e2[2]));
+    const float4 o = r.o;
+    const float pvx = d.y * e2.z - d.z * e2.y;
+    const float pvy = d.z * e2.x - d.x * e2.z;
+    const float pvz = d.x * e2.y - d.y * e2.x;
+    const float det = e1.x * pvx + e1.y * pvy + e1.z * pvz;
+    if (det == 0.0f) return false;
+    const float inv = __frcp_rn(det);
+    const float tvx = o.x - v0.x, tvy = o.y - v0.y, tvz = o.z - v0.z;
+    u = (tvx * pvx + tvy * pvy + tvz * pvz) * inv;
+    if (!(u >= 0.0f && u <= 1.0f)) return false;
+    const float qvx = tvy * e1.z - tvz * e1.y;
+    const float qvy = tvz * e1.x - tvx * e1.z;
+    const float qvz = tvx * e1.y - tvy * e1.x;
+    v = (d.x * qvx + d.y * qvy + d.z * qvz) * inv;
+    if (!(v >= 0.0f && u + v <= 1.0f)) return false;
+    t = (e2.x * qvx + e2.y * qvy + e2.z * qvz) * inv;
+    return t > o.w && t < r.best;
+}
+
+// Tests the first triangle of the pending group.  ANY: a hit ends the ray.
+template <bool ANY, typename X>
+__device__ __forceinline__ void test_one_triangle(RayState &r, X &x, const SceneRef &a, uint32_t *err) {
+    const uint32_t b = __ffs(r.t.hits) - 1u;
+    r.t.hits &= r.t.hits - 1u;
+    const uint32_t k = r.t.base + __popc(r.t.all & ((1u << b) - 1u));
+    if (!index_ok(k, a.n_tris, err)) return;
+    float u, v, t;
+    if (meet_triangle(r, x.d(), a, k, u, v, t)) {
+        r.best = t;
+        x.set_hit(u, v, k);
+        if (ANY) ray_stop(r);
+    }
+}
+
+template <typename X>
+__device__ __forceinline__ float4 ray_result(const RayState &r, const X &x, const SceneRef &a) {
+    const Hit h = x.hit();
+    if (h.k == kMiss) return make_float4(__int_as_float(0x7f800000), 0.0f, 0.0f, __uint_as_float(kMiss));
+    const float tr = refine_t(a, h.k, r.o, x.d());
+    const float id = __uint_as_float(__ldg(&a.tris[h.k].id));  // the triangle's number in the caller's soup
+    return make_float4(isfinite(tr) ? tr : r.best, h.u, h.v, id);
 }
 
 // The length-table update of one traced ray (Section 3.1.6), the arithmetic of
 // table_accumulate_kernel: a ray that hit adds trunc(clamp(t*|d|/E, 0, 64)*2^24)
 // and one count to the cell of its 20-bit compacted Aila code.
 __device__ __forceinline__ void accumulate_hit(unsigned long long *table, const QuantFrame &f, float invE,
-                                               float4 o, float4 d, float4 h) {
+                                               float4 o, float3 dir, float4 h) {
+    const float4 d = make_float4(dir.x, dir.y, dir.z, 0.0f);
     if (__float_as_uint(h.w) == kMiss || !isfinite(h.x)) return;
     uint32_t qo[3], qd[3];
     float dh[3];
@@ -308,31 +496,188 @@ __device__ __forceinline__ void accumulate_hit(unsigned long long *table, const 
     atomicAdd(table + 2 * (size_t)cell + 1, 1ull);
 }
 
-// One traversal step of a lane's ray: test one pending triangle, or (after
-// popping the next node group when the current one is used up) visit one
-// node.  Returns false once the ray is finished.  A stack that would
-// overflow records RR_DEVERR_TRACE_STACK and ends the ray as a miss.
-template <bool ANY>
-__device__ __forceinline__ bool ray_step(RayState &r, uint2 *stack, const SceneRef &sc, uint32_t *err) {
-    if (r.t_hits != 0u) {
-        test_one_triangle<ANY>(r, sc, err);
-        return true;
+// One traversal step of a warp's rays: every lane tests the first pending
+// triangle of its ray and, unless two triangle groups are still waiting after
+// it, visits one node (after popping the next node group when the current one
+// is used up).  Returns false for a lane without a ray or whose ray is
+// finished.  All lanes of the warp call it together; it brings them together
+// again before the node visit, which would otherwise be issued once for the
+// lanes that tested a triangle and once more for those that did not.  A stack
+// that would overflow records RR_DEVERR_TRACE_STACK and ends the ray as a miss.
+template <bool ANY, bool LEAN, int BLOCK>
+__device__ __forceinline__ bool ray_step(RayState &r, LaneExtra<LEAN, BLOCK> &x, bool live, uint2 *l_stack,
+                                         const SceneRef &sc, uint32_t *err, const uint8_t *s_oct) {
+    uint2 *s_stack = x.m.stack + x.at;  // entries BLOCK apart
+    bool more = live;
+    if (live && r.t.hits != 0u) {
+        test_one_triangle<ANY>(r, x, sc, err);
+        next_group(r, x);
     }
-    if (r.g_hits == 0u) {
-        if (r.sp == 0) return false;
-        const uint2 e = stack[--r.sp];
-        r.g_base = e.x;
-        r.g_hits = e.y & 0xFFu;
-        r.g_imask = (e.y >> 8) & 0xFFu;
+    __syncwarp();
+    bool visit = live && r.u_hits == 0u;
+    if (visit && (r.g_mask & 0xFFu) == 0u) {
+        if (r.sp == 0) {
+            visit = false;
+            more = r.t.hits != 0u;
+        } else {
+            --r.sp;
+            const uint2 e = r.sp < kSharedStack ? s_stack[r.sp * BLOCK] : l_stack[r.sp - kSharedStack];
+            r.g_base = e.x;
+            r.g_mask = e.y;
+        }
     }
-    if (!ray_visit_node(r, stack, sc, err)) {
-        atomicOr(err, RR_DEVERR_TRACE_STACK);
-        r.best_tri = kMiss;
-        r.g_hits = 0u;
-        r.t_hits = 0u;
-        r.sp = 0;
+    if (visit) {
+        const uint32_t node = take_child(r);
+        bool ok = index_ok(node, sc.n_nodes, err);
+        if ((r.g_mask & 0xFFu) != 0u) {
+            const uint2 e = make_uint2(r.g_base, r.g_mask);
+            if (r.sp < kSharedStack) {
+                s_stack[r.sp * BLOCK] = e;
+            } else if (r.sp < (int)kTraceStack) {
+                l_stack[r.sp - kSharedStack] = e;
+            } else {
+                atomicOr(err, RR_DEVERR_TRACE_STACK);
+                ok = false;
+            }
+            ++r.sp;
+        }
+        if (ok) {
+            const DevNode *np = sc.nodes + node;
+            const Words8 n0 = load256(np), n1 = load256(&np->qlo_x), n2 = load256(&np->qlo_z);
+            take_hits(r, x, n0, n2, hit_slots(r, node_slabs(r, n0, n1, n2)), s_oct);
+        } else {
+            x.set_hit(0.0f, 0.0f, kMiss);
+            ray_stop(r);
+        }
     }
-    return true;
+    return more;
+}
+
+// ------------------------------------------------------------------ four lanes to a ray
+//
+// Where a warp has few rays, the time is the latency of its longest ray: the
+// instructions of a step, at one warp's issue rate, and its loads.  Four lanes
+// then share a ray: each holds the whole ray state, tests two of a node's
+// eight slots and one of up to four pending triangles.  The triangles of a
+// group are taken four at a time in their order, and of equal distances the
+// first one wins, so the result is the one-lane traversal's.  All lanes of the
+// warp run the loop together.
+//
+// stack: the warp's shared stack rows (row e of the block's stack lies BLOCK
+// entries after row e - 1); the warp's eight rays divide the rows of its 32
+// lanes, 4 * kSharedStack = 32 entries each.
+static_assert(4 * kSharedStack >= (int)kTraceStack, "a ray's share of the warp's stack rows is too small");
+
+template <int BLOCK>
+__device__ __forceinline__ uint32_t quad_entry(uint32_t sp, uint32_t quad) {
+    return (sp >> 2) * BLOCK + (sp & 3u) * 8u + quad;
+}
+
+// One step: up to four pending triangles, or the next node.  Returns false
+// for the lanes of a ray that is finished (or of no ray).
+template <bool ANY, int BLOCK>
+__device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool live, uint2 *stack, const SceneRef &sc,
+                                          uint32_t *err, const uint8_t *s_oct) {
+    const uint32_t lane = threadIdx.x & 31u, quad = lane >> 2, j = lane & 3u;
+    const bool test = live && r.t.hits != 0u;
+    if (__any_sync(0xFFFFFFFFu, test)) {
+        float u = 0.0f, v = 0.0f, t = __int_as_float(0x7f800000);
+        uint32_t k = kMiss;
+        bool hit = false;
+        if (test) {
+            const uint32_t h0 = r.t.hits, h1 = h0 & (h0 - 1u), h2 = h1 & (h1 - 1u), h3 = h2 & (h2 - 1u);
+            const uint32_t mine = j == 0u ? h0 : j == 1u ? h1 : j == 2u ? h2 : h3;
+            if (mine != 0u) {
+                k = r.t.base + __popc(r.t.all & ((mine & (0u - mine)) - 1u));
+                if (index_ok(k, sc.n_tris, err)) hit = meet_triangle(r, x.d(), sc, k, u, v, t);
+                if (!hit) t = __int_as_float(0x7f800000);
+            }
+            r.t.hits = h3 & (h3 - 1u);
+            next_group(r, x);
+        }
+        const uint32_t hits = (__ballot_sync(0xFFFFFFFFu, hit) >> (4u * quad)) & 15u;
+        if (__any_sync(0xFFFFFFFFu, hit)) {
+            // the winning lane of the four: the nearest hit (ANY: the first), the
+            // first among equals
+            uint32_t win;
+            if (ANY) {
+                win = hits ? __ffs(hits) - 1u : 0u;
+            } else {
+                win = j;
+                float tw = t;
+#pragma unroll
+                for (int by = 1; by <= 2; by <<= 1) {
+                    const float to = __shfl_xor_sync(0xFFFFFFFFu, tw, by);
+                    const uint32_t wo = __shfl_xor_sync(0xFFFFFFFFu, win, by);
+                    if (to < tw || (to == tw && wo < win)) {
+                        tw = to;
+                        win = wo;
+                    }
+                }
+            }
+            const uint32_t from = 4u * quad + win;
+            const float tw = __shfl_sync(0xFFFFFFFFu, t, from), uw = __shfl_sync(0xFFFFFFFFu, u, from),
+                        vw = __shfl_sync(0xFFFFFFFFu, v, from);
+            const uint32_t kw = __shfl_sync(0xFFFFFFFFu, k, from);
+            if (hits != 0u) {
+                r.best = tw;
+                x.set_hit(uw, vw, kw);
+                if (ANY) ray_stop(r);
+            }
+        }
+    }
+    __syncwarp();
+    bool visit = live && r.t.hits == 0u, more = live;
+    if (visit && (r.g_mask & 0xFFu) == 0u) {
+        if (r.sp == 0) {
+            visit = false;
+            more = false;
+        } else {
+            --r.sp;
+            const uint2 e = stack[quad_entry<BLOCK>(r.sp, quad)];
+            r.g_base = e.x;
+            r.g_mask = e.y;
+        }
+    }
+    Words8 n0{}, n2{};
+    bool two[2] = {false, false};
+    if (visit) {
+        const uint32_t node = take_child(r);
+        visit = index_ok(node, sc.n_nodes, err);
+        if ((r.g_mask & 0xFFu) != 0u) {
+            if (r.sp < (int)kTraceStack) {
+                stack[quad_entry<BLOCK>(r.sp, quad)] = make_uint2(r.g_base, r.g_mask);  // the four lanes store the same
+            } else {
+                atomicOr(err, RR_DEVERR_TRACE_STACK);
+                visit = false;
+            }
+            ++r.sp;
+        }
+        if (visit) {
+            const DevNode *np = sc.nodes + node;
+            n0 = load256(np);
+            n2 = load256(&np->qlo_z);
+            const NodeSlabs s = node_slabs(r, n0, load256(&np->qlo_x), n2);
+            const uint32_t sel = 0x7540u | j;  // byte j, then the mantissa and exponent of 2^23
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const auto at = [&](uint32_t w, float b, float a) {
+                    return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), b, a);
+                };
+                const float t0 = max3f(at(s.nx[h], s.bx, s.ax), at(s.ny[h], s.by, s.ay),
+                                       fmaxf(at(s.nz[h], s.bz, s.az), r.o.w));
+                const float t1 = min3f(at(s.fx[h], s.bx, s.ax), at(s.fy[h], s.by, s.ay),
+                                       fminf(at(s.fz[h], s.bz, s.az), r.best));
+                two[h] = t0 <= t1;
+            }
+        } else {
+            x.set_hit(0.0f, 0.0f, kMiss);
+            ray_stop(r);
+        }
+    }
+    const uint32_t lo = __ballot_sync(0xFFFFFFFFu, two[0]), hi = __ballot_sync(0xFFFFFFFFu, two[1]);
+    if (visit) take_hits(r, x, n0, n2, ((lo >> (4u * quad)) & 15u) | (((hi >> (4u * quad)) & 15u) << 4), s_oct);
+    return more;
 }
 
 // Lanes refill from the queue once this many of a warp's 32 lanes are idle
@@ -340,56 +685,132 @@ __device__ __forceinline__ bool ray_step(RayState &r, uint2 *stack, const SceneR
 // lanes take consecutive queue positions together.
 constexpr uint32_t kRefillLanes = 8;
 
-// Resident blocks asked of the compiler: 36 warps per SM (nine 128-thread
-// blocks at 56 registers; the step loop keeps the ray's state and the refill
-// bookkeeping without spills).  Larger blocks round down to 32 warps.
-template <int BLOCK>
+// With the queue empty, a warp left with this many rays or fewer goes on with
+// four lanes to each: its longest rays decide when the launch ends (689,149
+// rays through the permutation, keys and sort included: 0.396 ms without the
+// hand-over, 0.362 ms with it).
+constexpr uint32_t kTailRays = 8;
+
+// Resident blocks asked of the compiler (see LaneExtra).
+template <bool MULTI, int BLOCK>
 constexpr int trace_min_blocks() {
-    return 1152 / BLOCK > 0 ? 1152 / BLOCK : 1;
+    return (trace_lean<MULTI, BLOCK>() ? 1152 : 1024) / BLOCK;
 }
 
 // Dynamic shared memory of the batch kernels: the scene of every segment, then
 // the segment offsets.
 inline size_t multi_smem(uint32_t n_segs) { return sizeof(SceneRef) * n_segs + sizeof(uint32_t) * (n_segs + 1); }
 
+// What the trace kernels share around the traversal.
+//
 // MULTI: rays of several scenes in one launch (a batch); each lane finds the
 // segment of its ray when it takes the ray and traces that segment's BVH
 // (and updates its table).  The segments' scenes sit in shared memory, so a
 // lane keeps only its segment number in registers during traversal.
-//
-// Each lane traces its own ray, one traversal step (a node or a triangle) per
-// loop iteration, so a warp spends an iteration on triangle tests only for as
-// long as some lane has a triangle left, and lanes whose ray has finished are
-// refilled from the queue (kRefillLanes at a time) instead of idling until the
-// warp's slowest ray is done.
-template <bool ACCUM, bool ANY, bool MULTI, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (trace_min_blocks<BLOCK>())) trace_kernel(TraceArgs a) {
-    extern __shared__ __align__(16) unsigned char s_dyn[];
-    SceneRef *s_sc = reinterpret_cast<SceneRef *>(s_dyn);
-    uint32_t *s_off = reinterpret_cast<uint32_t *>(s_sc + (MULTI ? a.n_segs : 0));
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t lanes_below = (1u << lane) - 1u;
+template <bool ACCUM, bool MULTI>
+struct TraceContext {
+    const TraceArgs &a;
+    SceneRef *s_sc;
+    uint32_t *s_off;
     // the table's quantisation frame is the same for the whole launch: it lives
     // in shared memory, not in every thread's registers during traversal
-    __shared__ QuantFrame s_frame;
-    __shared__ float s_invE;
-    uint2 stack[kTraceStack];
-    if (ACCUM && !MULTI && threadIdx.x == 0) {
-        s_frame = make_frame(a.tlo, a.thi);
-        s_invE = __fdiv_rn(1.0f, s_frame.E);
-    }
-    if (MULTI) {
-        for (uint32_t k = threadIdx.x; k <= a.n_segs; k += BLOCK) s_off[k] = a.seg_offsets[k];
-        for (uint32_t k = threadIdx.x; k < a.n_segs; k += BLOCK) {
-            const BatchScene *bs = a.segs + k;
-            s_sc[k].nodes = bs->nodes;
-            s_sc[k].tris = bs->tris;
-            s_sc[k].planes = bs->planes;
-            s_sc[k].n_nodes = bs->n_nodes;
-            s_sc[k].n_tris = bs->n_tris;
+    QuantFrame *s_frame;
+    float *s_invE;
+
+    // Called by every thread; the caller synchronises the block afterwards.
+    __device__ __forceinline__ void load() const {
+        if (ACCUM && !MULTI && threadIdx.x == 0) {
+            *s_frame = make_frame(a.tlo, a.thi);
+            *s_invE = __fdiv_rn(1.0f, s_frame->E);
+        }
+        if (MULTI) {
+            for (uint32_t k = threadIdx.x; k <= a.n_segs; k += blockDim.x) s_off[k] = a.seg_offsets[k];
+            for (uint32_t k = threadIdx.x; k < a.n_segs; k += blockDim.x) {
+                const BatchScene *bs = a.segs + k;
+                s_sc[k].nodes = bs->nodes;
+                s_sc[k].tris = bs->tris;
+                s_sc[k].n_nodes = bs->n_nodes;
+                s_sc[k].n_tris = bs->n_tris;
+            }
         }
     }
-    if (MULTI || ACCUM) __syncthreads();
+    __device__ __forceinline__ const SceneRef &scene(uint32_t seg) const { return MULTI ? s_sc[seg] : a.scene; }
+
+    // Queue position pos -> ray and segment.  false: not a position, or (an
+    // index buffer that is no permutation) no ray of the launch.
+    __device__ __forceinline__ bool find_ray(uint32_t pos, uint32_t &ray, uint32_t &seg) const {
+        if (pos >= a.n) return false;
+        const uint32_t i = a.order ? __ldg(a.order + pos) : pos;
+        if (i >= a.n) {  // not a permutation of [0, n): record and skip
+            atomicOr(a.err, RR_DEVERR_BAD_INDEX);
+            return false;
+        }
+        ray = i;
+        if (MULTI) {
+            // the last segment starting at or before i (empty segments share
+            // their start with the next one, which wins)
+            uint32_t lo = 0, hi = a.n_segs;
+            while (hi - lo > 1) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (s_off[mid] <= i)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            seg = lo;
+        }
+        return true;
+    }
+
+    template <typename X>
+    __device__ __forceinline__ void store(const RayState &r, const X &x, uint32_t ray, uint32_t seg) const {
+        const float4 h = ray_result(r, x, scene(seg));
+        a.hits[ray] = h;
+        if (ACCUM) {
+            if (MULTI) {
+                const BatchScene *bs = a.segs + seg;
+                if (bs->table) accumulate_hit(bs->table, bs->frame, bs->invE, r.o, x.d(), h);
+            } else if (a.table) {
+                accumulate_hit(a.table, *s_frame, *s_invE, r.o, x.d(), h);
+            }
+        }
+    }
+
+    // The last block to leave the launch resets the queue for the next one.
+    __device__ __forceinline__ void leave() const {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            const uint32_t prev = atomicAdd(a.queue + 1, 1u);
+            if (prev == gridDim.x - 1) {  // every block has stopped fetching
+                a.queue[0] = 0u;
+                a.queue[1] = 0u;
+            }
+        }
+    }
+};
+
+// Each lane traces its own ray, at most one triangle and one node per loop
+// iteration, and lanes whose ray has finished are refilled from the queue
+// (kRefillLanes at a time) instead of idling until the warp's slowest ray is
+// done.
+template <bool ACCUM, bool ANY, bool MULTI, int BLOCK>
+__global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) trace_kernel(TraceArgs a) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ QuantFrame s_frame;
+    __shared__ float s_invE;
+    constexpr bool LEAN = trace_lean<MULTI, BLOCK>();
+    __shared__ LaneMem<LEAN, BLOCK> s_lane;
+    SceneRef *s_sc = reinterpret_cast<SceneRef *>(s_dyn);
+    const TraceContext<ACCUM, MULTI> cx{a, s_sc, reinterpret_cast<uint32_t *>(s_sc + (MULTI ? a.n_segs : 0)), &s_frame,
+                                        &s_invE};
+    cx.load();
+    const uint8_t *s_oct = block_octant_table();
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t lanes_below = (1u << lane) - 1u;
+    LaneExtra<LEAN, BLOCK> x{s_lane, threadIdx.x, make_float3(0.0f, 0.0f, 0.0f), make_uint2(0u, 0u)};
+    uint2 l_stack[kTraceStack - kSharedStack];
     RayState r;
     uint32_t ray = 0, seg = 0;
     bool live = false, finished = false, exhausted = false;
@@ -397,71 +818,114 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<BLOCK>())) trace_kern
         const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !live);
         if ((uint32_t)__popc(idle) >= kRefillLanes) {
             if (finished) {  // the hits of the lanes whose rays finished
-                const SceneRef &sc = MULTI ? s_sc[seg] : a.scene;
-                const float4 h = ray_result(r, sc);
-                a.hits[ray] = h;
-                if (ACCUM) {
-                    if (MULTI) {
-                        const BatchScene *bs = a.segs + seg;
-                        if (bs->table) accumulate_hit(bs->table, bs->frame, bs->invE, r.o, r.d, h);
-                    } else if (a.table) {
-                        accumulate_hit(a.table, s_frame, s_invE, r.o, r.d, h);
-                    }
-                }
+                cx.store(r, x, ray, seg);
                 finished = false;
             }
-            if (exhausted) {
-                if (idle == 0xFFFFFFFFu) break;
-            } else {
+            if (!exhausted) {
                 // idle lanes take consecutive queue positions, in lane order
                 const uint32_t want = __popc(idle);
                 uint32_t base = 0;
                 if (lane == 0) base = atomicAdd(a.queue, want);
                 base = __shfl_sync(0xFFFFFFFFu, base, 0);
                 if (base + want >= a.n) exhausted = true;
-                if (!live) {
-                    const uint32_t pos = base + __popc(idle & lanes_below);
-                    if (pos < a.n) {
-                        const uint32_t i = a.order ? __ldg(a.order + pos) : pos;
-                        if (i >= a.n) {  // not a permutation of [0, n): record and skip
-                            atomicOr(a.err, RR_DEVERR_BAD_INDEX);
-                        } else {
-                            ray = i;
-                            if (MULTI) {
-                                // the last segment starting at or before i (empty
-                                // segments share their start with the next one, which wins)
-                                uint32_t lo = 0, hi = a.n_segs;
-                                while (hi - lo > 1) {
-                                    const uint32_t mid = (lo + hi) >> 1;
-                                    if (s_off[mid] <= i)
-                                        lo = mid;
-                                    else
-                                        hi = mid;
-                                }
-                                seg = lo;
-                            }
-                            ray_begin(r, MULTI ? s_sc[seg] : a.scene, __ldg(a.o_tmin + i), __ldg(a.d_tmax + i));
-                            live = true;
-                        }
-                    }
+                if (!live && cx.find_ray(base + __popc(idle & lanes_below), ray, seg)) {
+                    ray_begin(r, x, cx.scene(seg), __ldg(a.o_tmin + ray), __ldg(a.d_tmax + ray));
+                    live = true;
                 }
-                if (exhausted && __ballot_sync(0xFFFFFFFFu, live) == 0u) break;
+            }
+            if (exhausted && (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, live)) <= kTailRays) break;
+        }
+        const bool more = ray_step<ANY, LEAN, BLOCK>(r, x, live, l_stack, cx.scene(seg), a.err, s_oct);
+        finished = finished || (live && !more);
+        live = more;
+    }
+    // the tail: at most eight rays are left, four lanes take each
+    const uint32_t rays = __ballot_sync(0xFFFFFFFFu, live);
+    if (rays != 0u) {
+        const uint32_t quad = lane >> 2;
+        uint2 *stack = s_lane.stack + (threadIdx.x & ~31u);
+        // owners move their stacks to their ray's rows (read before any is written)
+        uint2 e[kSharedStack];
+#pragma unroll
+        for (int i = 0; i < kSharedStack; ++i) e[i] = s_lane.stack[i * BLOCK + threadIdx.x];
+        __syncwarp();
+        if (live) {
+            const uint32_t to = __popc(rays & lanes_below);
+#pragma unroll
+            for (int i = 0; i < kSharedStack; ++i)
+                if (i < r.sp) stack[quad_entry<BLOCK>(i, to)] = e[i];
+            for (int i = kSharedStack; i < r.sp; ++i) stack[quad_entry<BLOCK>(i, to)] = l_stack[i - kSharedStack];
+        }
+        __syncwarp();
+        // the lane whose ray this lane's four take over
+        uint32_t left = rays;
+        for (uint32_t q = 0; q < quad; ++q) left &= left - 1u;
+        const uint32_t from = left ? __ffs(left) - 1u : 0u;
+        RayState q;
+#define RR_TAKE(F) q.F = __shfl_sync(0xFFFFFFFFu, r.F, from);
+        RR_TAKE(o.x) RR_TAKE(o.y) RR_TAKE(o.z) RR_TAKE(o.w)
+        RR_TAKE(idx) RR_TAKE(idy) RR_TAKE(idz) RR_TAKE(negmask) RR_TAKE(best)
+        RR_TAKE(g_base) RR_TAKE(g_mask) RR_TAKE(t.base) RR_TAKE(t.hits) RR_TAKE(t.all)
+        RR_TAKE(u_hits) RR_TAKE(sp)
+#undef RR_TAKE
+        const uint32_t qray = __shfl_sync(0xFFFFFFFFu, ray, from), qseg = __shfl_sync(0xFFFFFFFFu, seg, from);
+        const LaneExtra<LEAN, BLOCK> owner{s_lane, (threadIdx.x & ~31u) + from, x.dir, x.second};
+        RegisterExtra qx{owner.d(), owner.hit(), owner.u()};
+        if (!LEAN) {
+            qx.dir = make_float3(__shfl_sync(0xFFFFFFFFu, x.dir.x, from), __shfl_sync(0xFFFFFFFFu, x.dir.y, from),
+                                 __shfl_sync(0xFFFFFFFFu, x.dir.z, from));
+            qx.second = make_uint2(__shfl_sync(0xFFFFFFFFu, x.second.x, from), __shfl_sync(0xFFFFFFFFu, x.second.y, from));
+        }
+        bool qlive = left != 0u;
+        while (__any_sync(0xFFFFFFFFu, qlive)) {
+            const bool more = quad_step<ANY, BLOCK>(q, qx, qlive, stack, cx.scene(qseg), a.err, s_oct);
+            if (qlive && !more && (lane & 3u) == 0u) cx.store(q, qx, qray, qseg);
+            qlive = more;
+        }
+    }
+    cx.leave();
+}
+
+// Few rays: four lanes to a ray from the start.
+template <bool ACCUM, bool ANY, bool MULTI, int BLOCK>
+__global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) trace_quad_kernel(TraceArgs a) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ QuantFrame s_frame;
+    __shared__ float s_invE;
+    __shared__ uint2 s_stack[kSharedStack * BLOCK];
+    SceneRef *s_sc = reinterpret_cast<SceneRef *>(s_dyn);
+    const TraceContext<ACCUM, MULTI> cx{a, s_sc, reinterpret_cast<uint32_t *>(s_sc + (MULTI ? a.n_segs : 0)), &s_frame,
+                                        &s_invE};
+    cx.load();
+    const uint8_t *s_oct = block_octant_table();
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u, quad = lane >> 2;
+    uint2 *stack = s_stack + (threadIdx.x & ~31u);
+    RayState r;
+    RegisterExtra x;
+    x.begin(make_float4(0.0f, 0.0f, 0.0f, 0.0f));
+    uint32_t ray = 0, seg = 0;
+    bool live = false, exhausted = false;
+    while (true) {
+        const uint32_t idle = __ballot_sync(0xFFFFFFFFu, !live);
+        if (!exhausted && idle != 0u) {
+            // idle quads take consecutive queue positions
+            const uint32_t want = (uint32_t)__popc(idle) >> 2;
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(a.queue, want);
+            base = __shfl_sync(0xFFFFFFFFu, base, 0);
+            if (base + want >= a.n) exhausted = true;
+            if (!live && cx.find_ray(base + ((uint32_t)__popc(idle & ((1u << (4u * quad)) - 1u)) >> 2), ray, seg)) {
+                ray_begin(r, x, cx.scene(seg), __ldg(a.o_tmin + ray), __ldg(a.d_tmax + ray));
+                live = true;
             }
         }
-        if (live && !ray_step<ANY>(r, stack, MULTI ? s_sc[seg] : a.scene, a.err)) {
-            live = false;
-            finished = true;
-        }
+        if (exhausted && __ballot_sync(0xFFFFFFFFu, live) == 0u) break;
+        const bool more = quad_step<ANY, BLOCK>(r, x, live, stack, cx.scene(seg), a.err, s_oct);
+        if (live && !more && (lane & 3u) == 0u) cx.store(r, x, ray, seg);
+        live = more;
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const uint32_t prev = atomicAdd(a.queue + 1, 1u);
-        if (prev == gridDim.x - 1) {  // every block has stopped fetching: reset for the next launch
-            a.queue[0] = 0u;
-            a.queue[1] = 0u;
-        }
-    }
+    cx.leave();
 }
 
 }  // namespace rr
@@ -470,33 +934,109 @@ using namespace rr;
 
 namespace {
 
+DevNode device_node(const RRNode8 &n) {
+    DevNode d{};
+    d.px = n.px;
+    d.py = n.py;
+    d.pz = n.pz;
+    d.masks = n.imask | n.valid << 8;
+    const uint32_t s[3] = {(uint32_t)n.ex << 23, (uint32_t)n.ey << 23, (uint32_t)n.ez << 23};
+    std::memcpy(&d.sx, &s[0], 4);
+    std::memcpy(&d.sy, &s[1], 4);
+    std::memcpy(&d.sz, &s[2], 4);
+    d.child_base = n.child_base;
+    std::memcpy(d.qlo_x, n.qlo_x, 8);
+    std::memcpy(d.qlo_y, n.qlo_y, 8);
+    std::memcpy(d.qlo_z, n.qlo_z, 8);
+    std::memcpy(d.qhi_x, n.qhi_x, 8);
+    std::memcpy(d.qhi_y, n.qhi_y, 8);
+    std::memcpy(d.qhi_z, n.qhi_z, 8);
+    d.tri_base = n.tri_base;
+    d.tribits = n.tribits;
+    return d;
+}
+
+RRNode8 host_node(const DevNode &d) {
+    RRNode8 n{};
+    n.px = d.px;
+    n.py = d.py;
+    n.pz = d.pz;
+    n.imask = (uint8_t)d.masks;
+    n.valid = d.masks >> 8;
+    uint32_t s[3];
+    std::memcpy(&s[0], &d.sx, 4);
+    std::memcpy(&s[1], &d.sy, 4);
+    std::memcpy(&s[2], &d.sz, 4);
+    n.ex = (uint8_t)(s[0] >> 23);
+    n.ey = (uint8_t)(s[1] >> 23);
+    n.ez = (uint8_t)(s[2] >> 23);
+    n.child_base = d.child_base;
+    std::memcpy(n.qlo_x, d.qlo_x, 8);
+    std::memcpy(n.qlo_y, d.qlo_y, 8);
+    std::memcpy(n.qlo_z, d.qlo_z, 8);
+    std::memcpy(n.qhi_x, d.qhi_x, 8);
+    std::memcpy(n.qhi_y, d.qhi_y, 8);
+    std::memcpy(n.qhi_z, d.qhi_z, 8);
+    n.tri_base = d.tri_base;
+    n.tribits = d.tribits;
+    return n;
+}
+
+DevTri device_tri(const RRTri &t, const float4 *planes) {
+    DevTri d;
+    const float w[16] = {t.v0_id.x, t.v0_id.y, t.v0_id.z, t.e1.x,      t.e1.y,      t.e1.z,      t.e2.x,      t.e2.y,
+                         t.e2.z,    t.v0_id.w, planes[0].x, planes[0].y, planes[0].z, planes[0].w, planes[1].x, planes[1].y};
+    std::memcpy(&d, w, sizeof(d));
+    return d;
+}
+
+void host_tri(const DevTri &d, const float *padding, RRTri *t, float4 *planes) {
+    float id;
+    std::memcpy(&id, &d.id, 4);
+    t->v0_id = make_float4(d.v0[0], d.v0[1], d.v0[2], id);
+    t->e1 = make_float4(d.e1[0], d.e1[1], d.e1[2], padding[0]);
+    t->e2 = make_float4(d.e2[0], d.e2[1], d.e2[2], padding[1]);
+    planes[0] = make_float4(d.nhi[0], d.nhi[1], d.nhi[2], d.nlo[0]);
+    planes[1] = make_float4(d.nlo[1], d.nlo[2], padding[2], padding[3]);
+}
+
+// Whether a triangle's unused words hold anything but zero bits.
+bool has_padding(const RRTri &t, const float4 &p1) {
+    const float w[4] = {t.e1.w, t.e2.w, p1.z, p1.w}, zero[4] = {};
+    return std::memcmp(w, zero, sizeof(w)) != 0;
+}
+
 // Uploads a host BVH into a new handle (synchronous).
 rr_status upload_bvh(const HostBVH &h, uint32_t n_tris, double seconds, const char *what, rr_bvh **out) {
     rr_bvh *b = new rr_bvh();
     cudaGetDevice(&b->device);
     b->nodes = nullptr;
     b->tris = nullptr;
-    b->planes = nullptr;
     b->n_nodes = (uint32_t)h.nodes.size();
     b->n_tris = n_tris;
     b->root_is_leaf = 0;
     b->root_leaf_ref = 0;
     cudaError_t e = cudaSuccess;
     if (b->n_nodes) {
-        e = lib_malloc(reinterpret_cast<void **>(&b->nodes), sizeof(RRNode8) * h.nodes.size());
-        if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void **>(&b->tris), sizeof(RRTri) * h.tris.size());
-        if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void **>(&b->planes), sizeof(float4) * h.planes.size());
+        std::vector<DevNode> nodes(h.nodes.size());
+        for (size_t i = 0; i < nodes.size(); ++i) nodes[i] = device_node(h.nodes[i]);
+        std::vector<DevTri> tris(h.tris.size());
+        for (size_t i = 0; i < tris.size(); ++i) tris[i] = device_tri(h.tris[i], &h.planes[2 * i]);
+        bool padded = false;
+        for (size_t i = 0; i < tris.size() && !padded; ++i) padded = has_padding(h.tris[i], h.planes[2 * i + 1]);
+        if (padded)
+            for (size_t i = 0; i < tris.size(); ++i)
+                for (float x : {h.tris[i].e1.w, h.tris[i].e2.w, h.planes[2 * i + 1].z, h.planes[2 * i + 1].w})
+                    b->padding.push_back(x);
+        e = lib_malloc(reinterpret_cast<void **>(&b->nodes), sizeof(DevNode) * nodes.size());
+        if (e == cudaSuccess) e = lib_malloc(reinterpret_cast<void **>(&b->tris), sizeof(DevTri) * tris.size());
         if (e == cudaSuccess)
-            e = cudaMemcpy(b->planes, h.planes.data(), sizeof(float4) * h.planes.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(b->nodes, h.nodes.data(), sizeof(RRNode8) * h.nodes.size(), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(b->tris, h.tris.data(), sizeof(RRTri) * h.tris.size(), cudaMemcpyHostToDevice);
+            e = cudaMemcpy(b->nodes, nodes.data(), sizeof(DevNode) * nodes.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemcpy(b->tris, tris.data(), sizeof(DevTri) * tris.size(), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
         cudaFree(b->nodes);
         cudaFree(b->tris);
-        cudaFree(b->planes);
         delete b;
         cudaGetLastError();
         return fail(e == cudaErrorMemoryAllocation ? RR_ERR_OOM : RR_ERR_CUDA, std::string(what) + ": upload failed");
@@ -554,11 +1094,14 @@ extern "C" rr_status rr_bvh_serialize(const rr_bvh *b, void *buf, size_t *bytes)
     h.planes.resize(2 * h.tris.size());
     cudaError_t e = cudaSuccess;
     if (b->n_nodes) {
-        e = cudaMemcpy(h.nodes.data(), b->nodes, sizeof(RRNode8) * h.nodes.size(), cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(h.tris.data(), b->tris, sizeof(RRTri) * h.tris.size(), cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(h.planes.data(), b->planes, sizeof(float4) * h.planes.size(), cudaMemcpyDeviceToHost);
+        std::vector<DevNode> nodes(h.nodes.size());
+        std::vector<DevTri> tris(h.tris.size());
+        e = cudaMemcpy(nodes.data(), b->nodes, sizeof(DevNode) * nodes.size(), cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(tris.data(), b->tris, sizeof(DevTri) * tris.size(), cudaMemcpyDeviceToHost);
+        const float none[4] = {};
+        for (size_t i = 0; i < nodes.size(); ++i) h.nodes[i] = host_node(nodes[i]);
+        for (size_t i = 0; i < tris.size(); ++i)
+            host_tri(tris[i], b->padding.empty() ? none : &b->padding[4 * i], &h.tris[i], &h.planes[2 * i]);
     }
     if (e != cudaSuccess) return fail_cuda(e, "rr_bvh_serialize: download");
     for (int c = 0; c < 3; ++c) {
@@ -588,7 +1131,6 @@ extern "C" rr_status rr_bvh_destroy(rr_bvh *b) {
     if (!b) return RR_OK;
     cudaFree(b->nodes);
     cudaFree(b->tris);
-    cudaFree(b->planes);
     delete b;
     return RR_OK;
 }
@@ -610,27 +1152,52 @@ extern "C" rr_status rr_bvh_aabb(const rr_bvh *b, float lo[3], float hi[3]) {
 
 namespace {
 
-template <bool ACC, bool ANY, bool MULTI, int BLOCK>
+// Launches of at most this many rays put four lanes to a ray: about as many as
+// the device then holds at once (152 SMs x 32 warps x 8).  A 4,097-ray bounce
+// takes 80 instead of 88 us; with 65,536 rays, two rounds of fours, it is
+// slower (172 against 148 us).
+constexpr uint32_t kQuadRays = 38912;
+
+template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
+void *trace_entry() {
+    return QUAD ? (void *)trace_quad_kernel<ACC, ANY, MULTI, BLOCK> : (void *)trace_kernel<ACC, ANY, MULTI, BLOCK>;
+}
+
+template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
 int trace_blocks_per_sm(size_t smem) {
     static int bps = 0;
     static size_t bps_smem = 0;
     if (bps == 0 || bps_smem != smem) {  // the batch kernels' shared memory varies with the segments
         int v = 0;
-        const cudaError_t e =
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, trace_kernel<ACC, ANY, MULTI, BLOCK>, BLOCK, smem);
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &v, trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>(), BLOCK, smem);
         bps = (e != cudaSuccess || v < 1) ? 1 : v;
         bps_smem = smem;
     }
     return bps;
 }
 
+template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
+void trace_enqueue_form(const TraceArgs &a, int sm_count, cudaStream_t s) {
+    const size_t smem = MULTI ? multi_smem(a.n_segs) : 0;
+    const uint32_t per_block = QUAD ? BLOCK / 4 : BLOCK;  // rays a block holds at a time
+    uint32_t grid = (uint32_t)sm_count * (uint32_t)trace_blocks_per_sm<QUAD, ACC, ANY, MULTI, BLOCK>(smem);
+    grid = std::max(1u, std::min(grid, (a.n + per_block - 1u) / per_block));
+    if (MULTI)  // static and dynamic shared memory together may pass the default 48 KB
+        cudaFuncSetAttribute(trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)multi_smem(kMaxBatchSegments));
+    if (QUAD)
+        trace_quad_kernel<ACC, ANY, MULTI, BLOCK><<<grid, BLOCK, smem, s>>>(a);
+    else
+        trace_kernel<ACC, ANY, MULTI, BLOCK><<<grid, BLOCK, smem, s>>>(a);
+}
+
 template <bool ACC, bool ANY, bool MULTI, int BLOCK>
 void trace_enqueue(const TraceArgs &a, int sm_count, cudaStream_t s) {
-    const size_t smem = MULTI ? multi_smem(a.n_segs) : 0;
-    const uint32_t want = (a.n + 31u) / 32u;  // warps that can get work
-    uint32_t grid = (uint32_t)sm_count * (uint32_t)trace_blocks_per_sm<ACC, ANY, MULTI, BLOCK>(smem);
-    grid = std::max(1u, std::min(grid, (want + BLOCK / 32 - 1) / (BLOCK / 32)));
-    trace_kernel<ACC, ANY, MULTI, BLOCK><<<grid, BLOCK, smem, s>>>(a);
+    if (a.n <= kQuadRays)
+        trace_enqueue_form<true, ACC, ANY, MULTI, BLOCK>(a, sm_count, s);
+    else
+        trace_enqueue_form<false, ACC, ANY, MULTI, BLOCK>(a, sm_count, s);
 }
 
 rr_status launch_trace(const rr_bvh *b, const float *o_tmin, const float *d_tmax, const uint32_t *order, uint32_t n,
@@ -652,9 +1219,8 @@ rr_status launch_trace(const rr_bvh *b, const float *o_tmin, const float *d_tmax
     if (!ds) return st;
     cudaStream_t s = as_stream(stream);
     TraceArgs a{};
-    a.scene.nodes = reinterpret_cast<const float4 *>(b->nodes);
-    a.scene.tris = reinterpret_cast<const float4 *>(b->tris);
-    a.scene.planes = b->planes;
+    a.scene.nodes = b->nodes;
+    a.scene.tris = b->tris;
     a.scene.n_nodes = b->n_nodes;
     a.scene.n_tris = b->n_tris;
     a.o_tmin = reinterpret_cast<const float4 *>(o_tmin);
