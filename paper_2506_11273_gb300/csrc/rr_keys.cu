@@ -469,7 +469,7 @@ extern "C" rr_status rr_key_sort(const float *o_tmin, const float *d_tmax, uint3
     note_launches(1);
     st = check_launch("rr_key_sort");
     if (st != RR_OK) return st;
-    return sort_enqueue_passes(keys_out, nullptr, perm_out, n, p->bits, radix_bits, workspace, a.err, ds->sm_count, s);
+    return sort_enqueue_passes(keys_out, nullptr, perm_out, n, p->bits, radix_bits, workspace, a.err, s);
 }
 
 extern "C" rr_status rr_length_table_create(const float lo[3], const float hi[3], rr_length_table **out,

@@ -6,6 +6,15 @@
 // published spans), and scatters through shared memory so that global writes
 // come out in runs.  Consecutive passes overlap launch and drain
 // (programmatic dependent launch).
+//
+// What bounds it: up to one wave of tiles the latency of a tile (time stamps in
+// the kernel, 1.2M 64-bit keys, us: loads 0.9, counts 1.0, ranking 2.3, scans
+// 1.0, look-back 1.7, shared scatter 1.8, writes 1.3, kernel boundary 1.2),
+// beyond that issue and latency together.  Hence tiles as small as one wave
+// allows (plan_sort), both scans behind one barrier, and 32-bit passes once a
+// 64-bit key's low half is used up.  Keys and sort together, before and after:
+// 4,097 32-bit keys 33 -> 23 us, 65,536 64-bit 71 -> 51, 689,149 32-bit 62 -> 56,
+// 1.2M 64-bit 134 -> 127, 2.07M 32-bit 108 -> 99, 8.3M 64-bit 617 -> 562.
 #include <algorithm>
 #include <mutex>
 
@@ -49,15 +58,42 @@ __device__ __forceinline__ void allow_dependent_launch() {
 }
 __device__ __forceinline__ void wait_for_prerequisite() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Keys per thread of a full-size tile.
 template <typename K>
-struct SortTile;
-template <>
-struct SortTile<uint32_t> {
-    static constexpr int kItems = 16;
+struct SortTile {
+    static constexpr int kItems = sizeof(K) == 8 ? 12 : 16;
 };
+
+// Look-back words: 64 bits, or 32 bits for sorts of fewer than 2^20 keys in at
+// most 2^11 tiles.
+template <typename W>
+struct LookbackWord;
 template <>
-struct SortTile<unsigned long long> {
-    static constexpr int kItems = 12;
+struct LookbackWord<unsigned long long> {
+    using W = unsigned long long;
+    static __device__ __forceinline__ W load(const W *p) { return ld_relaxed(p); }
+    static __device__ __forceinline__ void store(W *p, W v) { st_relaxed(p, v); }
+    static __device__ __forceinline__ W make(uint32_t start, uint32_t count) { return lookback_word(start, count); }
+    static __device__ __forceinline__ bool ready(W w) { return (w & kReady) != 0; }
+    static __device__ __forceinline__ uint32_t start(W w) { return (uint32_t)(w >> 32) & 0x7FFFFFFFu; }
+    static __device__ __forceinline__ uint32_t count(W w) { return (uint32_t)w; }
+};
+constexpr uint32_t kSmallSortKeys = 1u << 20;
+template <>
+struct LookbackWord<uint32_t> {
+    using W = uint32_t;
+    static __device__ __forceinline__ W load(const W *p) {
+        W v;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+        return v;
+    }
+    static __device__ __forceinline__ void store(W *p, W v) {
+        asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+    }
+    static __device__ __forceinline__ W make(uint32_t start, uint32_t count) { return 0x80000000u | start << 20 | count; }
+    static __device__ __forceinline__ bool ready(W w) { return (w >> 31) != 0; }
+    static __device__ __forceinline__ uint32_t start(W w) { return (w >> 20) & 0x7FFu; }
+    static __device__ __forceinline__ uint32_t count(W w) { return w & 0xFFFFFu; }
 };
 
 template <typename K>
@@ -80,26 +116,41 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t dg, uint32_t among) {
     return peers;
 }
 
-// Exclusive scan of one value per thread over the first `RADIX` threads
-// (threads beyond contribute zero).  Called by every thread of the block.
-template <int RADIX>
-__device__ __forceinline__ uint32_t scan_digits(uint32_t v, uint32_t *s_warp) {
+// Exclusive scans of COUNT values per thread over the first `RADIX` threads
+// (threads beyond contribute zero), together: one barrier.  Called by every
+// thread of the block.  s_warp: COUNT * kSortWarps words, 16-byte aligned, not
+// used by another scan of the block since the last barrier.
+template <int RADIX, int COUNT>
+__device__ __forceinline__ void scan_digits(uint32_t (&v)[COUNT], uint32_t *s_warp) {
+    static_assert(kSortWarps == 8, "two 16-byte reads cover the warp totals");
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    uint32_t x = v;
+    uint32_t x[COUNT];
+#pragma unroll
+    for (int q = 0; q < COUNT; ++q) x[q] = v[q];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-        if (lane >= (uint32_t)o) x += y;
+#pragma unroll
+        for (int q = 0; q < COUNT; ++q) {
+            const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x[q], o);
+            if (lane >= (uint32_t)o) x[q] += y;
+        }
     }
     if (RADIX > 32) {
-        if (lane == 31) s_warp[warp] = x;
+        if (lane == 31) {
+#pragma unroll
+            for (int q = 0; q < COUNT; ++q) s_warp[q * kSortWarps + warp] = x[q];
+        }
         __syncthreads();
-        uint32_t add = 0;
-        for (uint32_t w = 0; w < warp; ++w) add += s_warp[w];
-        __syncthreads();
-        x += add;
+#pragma unroll
+        for (int q = 0; q < COUNT; ++q) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(s_warp + q * kSortWarps),
+                        b = *reinterpret_cast<const uint4 *>(s_warp + q * kSortWarps + 4);
+            x[q] += (warp > 0 ? a.x : 0u) + (warp > 1 ? a.y : 0u) + (warp > 2 ? a.z : 0u) + (warp > 3 ? a.w : 0u) +
+                    (warp > 4 ? b.x : 0u) + (warp > 5 ? b.y : 0u) + (warp > 6 ? b.z : 0u);
+        }
     }
-    return x - v;
+#pragma unroll
+    for (int q = 0; q < COUNT; ++q) v[q] = x[q] - v[q];
 }
 
 // ------------------------------------------------------------------ upfront histograms
@@ -165,38 +216,40 @@ struct PassArgs {
     const K *keys_in;
     const uint32_t *vals_in;  // null on the first pass: the value is the input index
     K *keys_out;              // null: keys are not written
+    uint32_t *high_out;       // 64-bit keys, not null: the keys' high halves are written here instead
     uint32_t *vals_out;
     uint32_t n;
     uint32_t shift;
     uint32_t mask;
     const uint32_t *hist;     // RADIX counts of this pass's digit over all keys
-    unsigned long long *lookback;  // [tiles][RADIX] look-back words
+    void *lookback;           // [tiles][RADIX] look-back words, zero at the start
+    void *lookback_next;      // the words the next pass uses, cleared here (null: none, or clear already)
     uint32_t *tile_counter;
     uint32_t *err;
 };
 
 // Shared-memory layout of one digit pass.
-template <typename K, int RBITS>
+template <typename K, int RBITS, int ITEMS>
 struct PassSmem {
     static constexpr int RADIX = 1 << RBITS;
-    static constexpr int TILE = kSortBlock * SortTile<K>::kItems;
+    static constexpr int TILE = kSortBlock * ITEMS;
     // keys [TILE] | values [TILE] | per-warp counters [warps][RADIX] | tile-local
-    // digit starts [RADIX] | global base per digit [RADIX] | tile counts
-    // [RADIX] | misc [16]: [0] tile id, [8..15] scan scratch
+    // digit starts [RADIX] | global base per digit [RADIX] | tile counts [RADIX]
+    // | misc [24]: [0] tile id, [8..23] scan scratch
     static constexpr size_t bytes =
-        sizeof(K) * TILE + sizeof(uint32_t) * (TILE + kSortWarps * RADIX + 3 * RADIX + 16);
+        sizeof(K) * TILE + sizeof(uint32_t) * (TILE + kSortWarps * RADIX + 3 * RADIX + 24);
 };
-static_assert(PassSmem<unsigned long long, 8>::bytes <= 48 * 1024 && PassSmem<uint32_t, 8>::bytes <= 48 * 1024,
+static_assert(PassSmem<unsigned long long, 8, 12>::bytes <= 48 * 1024 && PassSmem<uint32_t, 8, 16>::bytes <= 48 * 1024,
               "a digit pass must fit the default dynamic shared-memory limit");
 
 // One tile of a digit pass.  FULL tiles skip every bounds check; only the
 // last tile of a pass can be partial.  LATE loads the values after the
 // ranking (their loads then overlap the look-back), which keeps the ranking's
 // registers low enough for four blocks per SM.
-template <typename K, int RBITS, bool FULL, bool LATE>
+template <typename K, int RBITS, int ITEMS, typename W, bool FULL, bool LATE>
 __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t tile, unsigned char *smem) {
+    using Word = LookbackWord<W>;
     constexpr int RADIX = 1 << RBITS;
-    constexpr int ITEMS = SortTile<K>::kItems;
     constexpr int TILE = kSortBlock * ITEMS;
     constexpr int WTILE = 32 * ITEMS;
     K *s_keys = reinterpret_cast<K *>(smem);
@@ -210,6 +263,7 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t base = tile * TILE;
     const uint32_t wbase = base + warp * WTILE;
+    const auto row = [&](uint32_t t) { return static_cast<W *>(a.lookback) + (size_t)t * RADIX + tid; };
 
     K k[ITEMS];
     uint32_t v[ITEMS], r[ITEMS];
@@ -224,14 +278,18 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
             if (!LATE) v[j] = 0;
         }
     }
+    // while the keys arrive: the pass's digit counts, and the next pass's words cleared
+    const uint32_t total = tid < RADIX ? a.hist[tid] : 0u;
+    if (a.lookback_next && tid < RADIX) static_cast<W *>(a.lookback_next)[(size_t)tile * RADIX + tid] = 0;
     // The tile's digit counts, published before the ranking so that later
-    // tiles looking back wait on this tile's loads only, not on its ranking.
+    // tiles looking back wait on this tile's loads only, not on its ranking
+    // (counts taken from the ranking instead: 1.2M 64-bit keys 0.137 -> 0.151 ms).
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j)
         if (FULL || wbase + j * 32 + lane < a.n) atomicAdd(&s_cnt[digit_of(k[j], a.shift, a.mask)], 1u);
     __syncthreads();
     const uint32_t cnt = tid < RADIX ? s_cnt[tid] : 0u;
-    if (tid < RADIX) st_relaxed(a.lookback + (size_t)tile * RADIX + tid, lookback_word(tile, cnt));
+    if (tid < RADIX) Word::store(row(tile), Word::make(tile, cnt));
 
     // stable rank inside the warp: items in index order (j, then lane).  The
     // peer masks of every row are independent; only the per-digit counters chain.
@@ -261,20 +319,25 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
         }
     }
 
-    // per digit: prefix over warps
+    // per digit: prefix over warps; digit starts in the output and in the tile
     if (tid < RADIX) {
         uint32_t acc = 0;
 #pragma unroll
-        for (int w = 0; w < kSortWarps; ++w) {
-            const uint32_t c = s_wh[w * RADIX + tid];
-            s_wh[w * RADIX + tid] = acc;
-            acc += c;
+        for (int w = 0; w < kSortWarps; w += 4) {
+            uint32_t c[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[q] = s_wh[(w + q) * RADIX + tid];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                s_wh[(w + q) * RADIX + tid] = acc;
+                acc += c[q];
+            }
         }
     }
-    const uint32_t dstart = scan_digits<RADIX>(tid < RADIX ? a.hist[tid] : 0u, s_misc + 8);
-    const uint32_t lstart = scan_digits<RADIX>(cnt, s_misc + 8);
-    uint32_t excl = 0;
+    uint32_t starts[2] = {total, cnt};
+    scan_digits<RADIX>(starts, s_misc + 8);
     if (tid < RADIX) {
+        uint32_t excl = 0;
         if (tile > 0) {
             // decoupled look-back by pointer jumping: add the span the nearest
             // uncovered predecessor has published and continue before its
@@ -283,8 +346,8 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
             // every tile of the pass runs at the same time.
             uint32_t start = tile, sum = cnt, spins = 0;
             while (start > 0) {
-                const unsigned long long w = ld_relaxed(a.lookback + (size_t)(start - 1) * RADIX + tid);
-                if (!(w & kReady)) {
+                const W w = Word::load(row(start - 1));
+                if (!Word::ready(w)) {
                     if (++spins > kSpinLimit) {
                         atomicOr(a.err, RR_DEVERR_LOOKBACK_TIMEOUT);
                         break;
@@ -292,14 +355,14 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
                     __nanosleep(32);
                     continue;
                 }
-                sum += (uint32_t)w;
-                start = (uint32_t)(w >> 32) & 0x7FFFFFFFu;
-                st_relaxed(a.lookback + (size_t)tile * RADIX + tid, lookback_word(start, sum));
+                sum += Word::count(w);
+                start = Word::start(w);
+                Word::store(row(tile), Word::make(start, sum));
             }
             excl = sum - cnt;
         }
-        s_lstart[tid] = lstart;
-        s_gbase[tid] = dstart + excl - lstart;
+        s_lstart[tid] = starts[1];
+        s_gbase[tid] = starts[0] + excl - starts[1];
     }
     __syncthreads();
 
@@ -315,33 +378,32 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
     }
     __syncthreads();
     // global writes in tile order: runs of equal digits land contiguously
+    const auto put = [&](uint32_t i) {
+        const K key = s_keys[i];
+        const uint32_t gpos = s_gbase[digit_of(key, a.shift, a.mask)] + i;
+        if (!index_ok(gpos, a.n, a.err)) return;
+        if (sizeof(K) == 8 && a.high_out)
+            a.high_out[gpos] = (uint32_t)((unsigned long long)key >> 32);
+        else if (a.keys_out)
+            a.keys_out[gpos] = key;
+        a.vals_out[gpos] = s_vals[i];
+    };
     if (FULL) {
 #pragma unroll
-        for (int j = 0; j < ITEMS; ++j) {
-            const uint32_t i = j * kSortBlock + tid;
-            const K key = s_keys[i];
-            const uint32_t gpos = s_gbase[digit_of(key, a.shift, a.mask)] + i;
-            if (!index_ok(gpos, a.n, a.err)) continue;
-            if (a.keys_out) a.keys_out[gpos] = key;
-            a.vals_out[gpos] = s_vals[i];
-        }
+        for (int j = 0; j < ITEMS; ++j) put(j * kSortBlock + tid);
     } else {
         const uint32_t tile_n = min((uint32_t)TILE, a.n - base);
-        for (uint32_t i = tid; i < tile_n; i += kSortBlock) {
-            const K key = s_keys[i];
-            const uint32_t gpos = s_gbase[digit_of(key, a.shift, a.mask)] + i;
-            if (!index_ok(gpos, a.n, a.err)) continue;
-            if (a.keys_out) a.keys_out[gpos] = key;
-            a.vals_out[gpos] = s_vals[i];
-        }
+        for (uint32_t i = tid; i < tile_n; i += kSortBlock) put(i);
     }
 }
 
 // MINB blocks per SM: 3 for passes of one wave or less (shortest tile
-// latency), 4 with late values for longer passes (more tiles in flight).
-template <typename K, int RBITS, int MINB>
+// latency), 4 with late values for longer passes (more tiles in flight: 506
+// tiles of 2.07M 32-bit keys, which three blocks per SM would run as one full
+// and one nearly empty wave, 105 -> 99 us for keys and sort).
+template <typename K, int RBITS, int ITEMS, typename W, int MINB>
 __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> a) {
-    using L = PassSmem<K, RBITS>;
+    using L = PassSmem<K, RBITS, ITEMS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *s_wh = reinterpret_cast<uint32_t *>(smem_raw + sizeof(K) * L::TILE) + L::TILE;
     uint32_t *s_cnt = s_wh + kSortWarps * L::RADIX + 2 * L::RADIX;
@@ -354,9 +416,9 @@ __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> 
     __syncthreads();
     const uint32_t tile = s_misc[0];
     if ((tile + 1) * (uint32_t)L::TILE <= a.n)
-        onesweep_tile<K, RBITS, true, (MINB > 3)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, true, (MINB > 3)>(a, tile, smem_raw);
     else
-        onesweep_tile<K, RBITS, false, (MINB > 3)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, false, (MINB > 3)>(a, tile, smem_raw);
 }
 
 // ------------------------------------------------------------------ local (segment) sort
@@ -421,8 +483,9 @@ __global__ void __launch_bounds__(kSortBlock) segment_sort_kernel(const K *__res
                 cnt += c;
             }
         }
-        const uint32_t start = scan_digits<RADIX>(cnt, s_scan);
-        if (tid < RADIX) s_dstart[tid] = start;
+        uint32_t start[1] = {cnt};
+        scan_digits<RADIX>(start, s_scan);
+        if (tid < RADIX) s_dstart[tid] = start[0];
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < ITEMS; ++j) {
@@ -488,26 +551,60 @@ static cudaError_t dispatch_segment_sort(const K *ki, K *ko, uint32_t *perm, uin
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct SortPlan {
-    uint32_t passes, radix, tiles, kb;
+    uint32_t passes, radix, kb;
+    uint32_t items;   // keys per thread of a pass over kb-byte keys
+    uint32_t tiles;   // its tiles
+    uint32_t wb;      // bytes of a look-back word
+    uint32_t regions; // sets of look-back words: a pass clears the set of the pass after it
     size_t off_hist, off_counters, off_lookback, off_keys_a, off_keys_b, off_vals, total;
 };
 
+// Tiles of a pass that fit on the device at three blocks per SM (152 SMs).
+constexpr uint32_t kWaveTiles = 456;
+
+constexpr uint32_t full_items(uint32_t kb) {
+    return kb == 8 ? SortTile<unsigned long long>::kItems : SortTile<uint32_t>::kItems;
+}
+
 // Workspace layout: digit counts [pass][radix], tile counters [pass],
-// 64-bit look-back words [pass][tile][radix], two key buffers, one value buffer.
+// look-back words, two key buffers, one value buffer.  The look-back part has
+// room for a 64-bit word per pass, full-size tile and digit; two sets of words
+// are used in turn.
+//
+// Tile size: the time of a pass of one wave is the latency of one tile, most
+// of it proportional to the keys of a thread (ranking, scatter), so the keys
+// are spread over as many tiles as still run at once: 4 keys per thread, then
+// 8, 12 and (32-bit keys) 16.  (64-bit words would not fit the smallest tiles
+// into the workspace, hence the 32-bit ones.)
 constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits) {
     SortPlan p{};
     p.passes = (bits + radix_bits - 1) / radix_bits;
     p.radix = 1u << radix_bits;
     p.kb = bits > 32 ? 8u : 4u;
-    const uint32_t tile = kSortBlock * (bits > 32 ? SortTile<unsigned long long>::kItems : SortTile<uint32_t>::kItems);
-    p.tiles = (n + tile - 1) / tile;
+    const uint32_t tile = kSortBlock * full_items(p.kb);
+    const uint32_t full_tiles = (n + tile - 1) / tile;
+    p.items = full_items(p.kb);
+    p.tiles = full_tiles;
+    p.wb = 8;
+    p.regions = p.passes > 1 ? 2u : 1u;
+    for (uint32_t items = 4; items < full_items(p.kb); items += 4) {
+        const uint32_t wb = items < 12 ? 4u : 8u;
+        const uint32_t tiles = (n + kSortBlock * items - 1) / (kSortBlock * items);
+        if ((wb == 4 && n >= kSmallSortKeys) || tiles > kWaveTiles ||
+            (uint64_t)wb * p.regions * tiles > 8ull * p.passes * full_tiles)
+            continue;
+        p.items = items;
+        p.tiles = tiles;
+        p.wb = wb;
+        break;
+    }
     size_t off = 0;
     p.off_hist = off;
     off = align256(off + sizeof(uint32_t) * p.passes * p.radix);
     p.off_counters = off;
     off = align256(off + sizeof(uint32_t) * p.passes);
     p.off_lookback = off;
-    off = align256(off + sizeof(unsigned long long) * (size_t)p.passes * p.tiles * p.radix);
+    off = align256(off + sizeof(unsigned long long) * (size_t)p.passes * full_tiles * p.radix);
     p.off_keys_a = off;
     off = align256(off + (size_t)p.kb * n);
     p.off_keys_b = off;
@@ -518,28 +615,40 @@ constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits) {
     return p;
 }
 
-template <typename K, int RBITS>
-static size_t pass_smem() {
-    return PassSmem<K, RBITS>::bytes;
-}
+// 16-byte words of a plan's look-back words, which start at zero.
+constexpr size_t lookback_uint4(const SortPlan &p) { return (size_t)p.regions * p.tiles * p.radix * p.wb / 16; }
 
 // One digit pass, launched so that it may start while the kernel before it
 // drains (programmatic dependent launch; the pass waits in the kernel).
-// Passes of at least two waves at four blocks per SM take the four-block form.
-template <typename K, int RBITS>
-static cudaError_t launch_pass(const PassArgs<K> &a, uint32_t tiles, int sm_count, cudaStream_t s) {
+template <typename K, int RBITS, int ITEMS, typename W, int MINB>
+static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tiles);
+    cfg.gridDim = dim3((a.n + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS));
     cfg.blockDim = dim3(kSortBlock);
-    cfg.dynamicSmemBytes = pass_smem<K, RBITS>();
+    cfg.dynamicSmemBytes = PassSmem<K, RBITS, ITEMS>::bytes;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (tiles >= 8u * (uint32_t)sm_count) return cudaLaunchKernelEx(&cfg, onesweep_kernel<K, RBITS, 4>, a);
-    return cudaLaunchKernelEx(&cfg, onesweep_kernel<K, RBITS, 3>, a);
+    return cudaLaunchKernelEx(&cfg, onesweep_kernel<K, RBITS, ITEMS, W, MINB>, a);
+}
+
+// The pass in the plan's tile size (for 64-bit plans also the passes over the
+// 32-bit high halves).  Full-size passes of more than one wave take the
+// four-block form.
+template <typename K, int RBITS>
+static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaStream_t s) {
+    using W64 = unsigned long long;
+    if (pl.items == 4) return launch_pass<K, RBITS, 4, uint32_t, 3>(a, s);
+    if (pl.items == 8) return launch_pass<K, RBITS, 8, uint32_t, 3>(a, s);
+    const uint32_t tiles12 = (a.n + kSortBlock * 12 - 1) / (kSortBlock * 12);
+    if (tiles12 <= kWaveTiles && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
+    constexpr int FULL = SortTile<K>::kItems;
+    const uint32_t tiles = (a.n + kSortBlock * FULL - 1) / (kSortBlock * FULL);
+    if (tiles > kWaveTiles) return launch_pass<K, RBITS, FULL, W64, 4>(a, s);
+    return launch_pass<K, RBITS, FULL, W64, 3>(a, s);
 }
 
 // The counting stage of a sort: the digit counts of every pass start at zero
@@ -550,10 +659,8 @@ static cudaError_t enqueue_count(const SortPlan &pl, const K *keys_in, uint32_t 
                                  uint32_t *zero_err, int sm_count, cudaStream_t s) {
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws + pl.off_hist);
     uint32_t *counters = reinterpret_cast<uint32_t *>(ws + pl.off_counters);
-    unsigned long long *lookback = reinterpret_cast<unsigned long long *>(ws + pl.off_lookback);
     cudaError_t e = cudaMemsetAsync(hist, 0, sizeof(uint32_t) * pl.passes * pl.radix, s);
     if (e != cudaSuccess) return e;
-    const size_t zero_count = (size_t)pl.passes * pl.tiles * pl.radix / 2;  // uint4 = two words
     const uint32_t per_block = kSortBlock * 4u;
     // counting-pass grid: two blocks per SM up to ~2M keys, then one block per
     // 8 rounds of keys up to eight per SM (more blocks in flight hide the
@@ -562,24 +669,29 @@ static cudaError_t enqueue_count(const SortPlan &pl, const K *keys_in, uint32_t 
     const uint32_t hist_blocks = std::max(
         1u, std::min({(n + per_block - 1) / per_block, std::max(2u * sms, n / (8u * per_block)), 8u * sms}));
     sort_histogram_kernel<K, RBITS><<<hist_blocks, kSortBlock, 0, s>>>(
-        keys_in, n, bits, pl.passes, hist, reinterpret_cast<uint4 *>(lookback), zero_count, counters, zero_err);
+        keys_in, n, bits, pl.passes, hist, reinterpret_cast<uint4 *>(ws + pl.off_lookback), lookback_uint4(pl), counters,
+        zero_err);
     note_launches(1);
     return cudaGetLastError();
 }
 
 // The digit passes of a sort whose counting stage has run (by enqueue_count
 // or fused into the key kernel): one onesweep kernel per pass.  Allocates
-// nothing.
+// nothing.  When the sorted keys are not wanted, a 64-bit sort drops the low
+// halves once their digits are used up, and the passes that are left move
+// 32-bit keys.
 template <typename K, int RBITS>
 static cudaError_t enqueue_passes(const SortPlan &pl, const K *keys_in, K *keys_out, uint32_t *perm_out,
-                                  uint32_t n, uint32_t bits, unsigned char *ws, uint32_t *err, int sm_count,
+                                  uint32_t n, uint32_t bits, unsigned char *ws, uint32_t *err,
                                   cudaStream_t s) {
     uint32_t *hist = reinterpret_cast<uint32_t *>(ws + pl.off_hist);
     uint32_t *counters = reinterpret_cast<uint32_t *>(ws + pl.off_counters);
-    unsigned long long *lookback = reinterpret_cast<unsigned long long *>(ws + pl.off_lookback);
     K *keys_a = reinterpret_cast<K *>(ws + pl.off_keys_a);
     K *keys_b = reinterpret_cast<K *>(ws + pl.off_keys_b);
     uint32_t *vals_ws = reinterpret_cast<uint32_t *>(ws + pl.off_vals);
+    const size_t region = (size_t)pl.tiles * pl.radix * pl.wb;
+    constexpr uint32_t kLowPasses = 32 / RBITS;  // passes over the low half of a 64-bit key
+    const uint32_t drop = sizeof(K) == 8 && !keys_out && pl.passes > kLowPasses ? kLowPasses - 1 : ~0u;
     const K *kin = keys_in;
     const uint32_t *vin = nullptr;
     for (uint32_t p = 0; p < pl.passes; ++p) {
@@ -590,20 +702,36 @@ static cudaError_t enqueue_passes(const SortPlan &pl, const K *keys_in, K *keys_
         else
             kout = final_slot ? (keys_out ? keys_out : keys_b) : keys_a;
         uint32_t *vout = final_slot ? perm_out : vals_ws;
-        PassArgs<K> a;
-        a.keys_in = kin;
-        a.vals_in = vin;
-        a.keys_out = kout;
-        a.vals_out = vout;
-        a.n = n;
-        a.shift = p * RBITS;
         const uint32_t nb = std::min<uint32_t>(RBITS, bits - p * RBITS);
-        a.mask = (1u << nb) - 1u;
-        a.hist = hist + p * pl.radix;
-        a.lookback = lookback + (size_t)p * pl.tiles * pl.radix;
-        a.tile_counter = counters + p;
-        a.err = err;
-        const cudaError_t e = launch_pass<K, RBITS>(a, pl.tiles, sm_count, s);
+        const auto fill = [&](auto &a) {
+            a.vals_in = vin;
+            a.vals_out = vout;
+            a.n = n;
+            a.mask = (1u << nb) - 1u;
+            a.hist = hist + p * pl.radix;
+            a.lookback = ws + pl.off_lookback + (p & 1u) * region;
+            // the words of the pass before this one become the next one's
+            a.lookback_next = p > 0 && p + 1 < pl.passes ? ws + pl.off_lookback + ((p + 1) & 1u) * region : nullptr;
+            a.tile_counter = counters + p;
+            a.err = err;
+        };
+        cudaError_t e;
+        if (p > drop && drop != ~0u) {
+            PassArgs<uint32_t> a{};
+            fill(a);
+            a.keys_in = reinterpret_cast<const uint32_t *>(kin);
+            a.keys_out = reinterpret_cast<uint32_t *>(kout);
+            a.shift = p * RBITS - 32;
+            e = dispatch_pass<uint32_t, RBITS>(pl, a, s);
+        } else {
+            PassArgs<K> a{};
+            fill(a);
+            a.keys_in = kin;
+            a.keys_out = kout;
+            a.high_out = p == drop ? reinterpret_cast<uint32_t *>(kout) : nullptr;
+            a.shift = p * RBITS;
+            e = dispatch_pass<K, RBITS>(pl, a, s);
+        }
         if (e != cudaSuccess) return e;
         kin = kout;
         vin = vout;
@@ -621,7 +749,7 @@ static cudaError_t enqueue_sort(const SortPlan &pl, const K *keys_in, K *keys_ou
                                 int sm_count, cudaStream_t s) {
     const cudaError_t e = enqueue_count<K, RBITS>(pl, keys_in, n, bits, ws, zero_err, sm_count, s);
     if (e != cudaSuccess) return e;
-    return enqueue_passes<K, RBITS>(pl, keys_in, keys_out, perm_out, n, bits, ws, err, sm_count, s);
+    return enqueue_passes<K, RBITS>(pl, keys_in, keys_out, perm_out, n, bits, ws, err, s);
 }
 
 template <typename K, int RBITS>
@@ -660,28 +788,28 @@ SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits
     t.hist = reinterpret_cast<uint32_t *>(ws + pl.off_hist);
     t.counters = reinterpret_cast<uint32_t *>(ws + pl.off_counters);
     t.zero_words = reinterpret_cast<uint4 *>(ws + pl.off_lookback);
-    t.zero_count = (size_t)pl.passes * pl.tiles * pl.radix / 2;
+    t.zero_count = lookback_uint4(pl);
     t.passes = pl.passes;
     t.radix_bits = radix_bits;
     return t;
 }
 
 rr_status sort_enqueue_passes(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
-                              uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s) {
+                              uint32_t radix_bits, void *workspace, uint32_t *err, cudaStream_t s) {
     const SortPlan pl = plan_sort(n, bits, radix_bits);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     cudaError_t e;
     if (pl.kb == 4) {
         const uint32_t *ki = static_cast<const uint32_t *>(keys_in);
         uint32_t *ko = static_cast<uint32_t *>(keys_out);
-        e = radix_bits == 8 ? enqueue_passes<uint32_t, 8>(pl, ki, ko, perm_out, n, bits, ws, err, sm_count, s)
-                            : enqueue_passes<uint32_t, 4>(pl, ki, ko, perm_out, n, bits, ws, err, sm_count, s);
+        e = radix_bits == 8 ? enqueue_passes<uint32_t, 8>(pl, ki, ko, perm_out, n, bits, ws, err, s)
+                            : enqueue_passes<uint32_t, 4>(pl, ki, ko, perm_out, n, bits, ws, err, s);
     } else {
         const unsigned long long *ki = static_cast<const unsigned long long *>(keys_in);
         unsigned long long *ko = static_cast<unsigned long long *>(keys_out);
         e = radix_bits == 8
-                ? enqueue_passes<unsigned long long, 8>(pl, ki, ko, perm_out, n, bits, ws, err, sm_count, s)
-                : enqueue_passes<unsigned long long, 4>(pl, ki, ko, perm_out, n, bits, ws, err, sm_count, s);
+                ? enqueue_passes<unsigned long long, 8>(pl, ki, ko, perm_out, n, bits, ws, err, s)
+                : enqueue_passes<unsigned long long, 4>(pl, ki, ko, perm_out, n, bits, ws, err, s);
     }
     if (e != cudaSuccess) return fail_cuda(e, "sort passes");
     if (fault_fires(Fault::Launch)) return fail(RR_ERR_CUDA, "sort passes: injected launch failure");
@@ -778,7 +906,7 @@ extern "C" rr_status rr_selftest_lookback_timeout(void *stream) {
     using K = uint32_t;
     constexpr uint32_t tile = kSortBlock * SortTile<K>::kItems;
     const uint32_t n = 2 * tile;
-    const SortPlan pl = plan_sort(n, 8, 8);
+    const SortPlan pl = plan_sort(n, 8, 8);  // (its full-size tile form is run here whatever the plan prefers)
     unsigned char *ws = nullptr;
     K *keys = nullptr, *keys_out = nullptr;
     uint32_t *perm = nullptr;
@@ -793,7 +921,7 @@ extern "C" rr_status rr_selftest_lookback_timeout(void *stream) {
     uint32_t *counter = reinterpret_cast<uint32_t *>(ws + pl.off_counters);
     if (e == cudaSuccess) e = cudaMemcpyAsync(counter, &one, sizeof(one), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
-        PassArgs<K> a;
+        PassArgs<K> a{};
         a.keys_in = keys;
         a.vals_in = nullptr;
         a.keys_out = keys_out;
@@ -802,10 +930,11 @@ extern "C" rr_status rr_selftest_lookback_timeout(void *stream) {
         a.shift = 0;
         a.mask = 0xFFu;
         a.hist = reinterpret_cast<const uint32_t *>(ws + pl.off_hist);
-        a.lookback = reinterpret_cast<unsigned long long *>(ws + pl.off_lookback);
+        a.lookback = ws + pl.off_lookback;
         a.tile_counter = counter;
         a.err = error_word(ds, s);
-        onesweep_kernel<K, 8, 3><<<1, kSortBlock, pass_smem<K, 8>(), s>>>(a);
+        onesweep_kernel<K, 8, SortTile<K>::kItems, unsigned long long, 3>
+            <<<1, kSortBlock, PassSmem<K, 8, SortTile<K>::kItems>::bytes, s>>>(a);
         note_launches(1);
         e = cudaGetLastError();
     }
