@@ -94,11 +94,11 @@ rr_status enqueue_batch(rr_batch *b, const float *o, const float *d, float *hits
         return launch_trace_batch(b->d_segs, b->d_offsets, b->n_fronts, o, d, nullptr, b->n_total, hits,
                                   accumulating(b), c.trace_block, b->queue, err, s);
     rr_status st = launch_keys_batch(b->d_segs, b->d_offsets, b->n_fronts, run_layout(b, c), run_tsrc(b, c), b->ratio,
-                                     c.key_bits,
-                                     b->seg_bits, o, d, b->n_total, b->keys, s);
+                                     c.key_bits, b->seg_bits, o, d, b->n_total, b->keys, c.radix_bits, b->sort_ws,
+                                     sm_count, s);
     if (st != RR_OK) return st;
-    st = sort_enqueue(b->keys, nullptr, perm, b->n_total, c.key_bits + b->seg_bits, c.radix_bits, b->sort_ws, err,
-                      sm_count, s);
+    st = sort_enqueue_passes(b->keys, nullptr, perm, b->n_total, c.key_bits + b->seg_bits, c.radix_bits, b->sort_ws,
+                             err, s);
     if (st != RR_OK) return st;
     return launch_trace_batch(b->d_segs, b->d_offsets, b->n_fronts, o, d, perm, b->n_total, hits, accumulating(b),
                               c.trace_block, b->queue, err, s);

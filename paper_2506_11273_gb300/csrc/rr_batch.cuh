@@ -26,11 +26,13 @@ cudaError_t launch_batch_frames(BatchScene *segs, const float *boxes, uint32_t n
 
 // Keys of every ray of a batch: segment s in the bits above key_bits, the
 // wavefront's own key (layout, estimate) below.  keys: u32 when
-// key_bits + seg_bits <= 32, else u64.
+// key_bits + seg_bits <= 32, else u64.  The counting stage of their sort with
+// radix_bits-bit digits is done on the way (sort_workspace: as for rr_sort);
+// sort_enqueue_passes follows.
 rr_status launch_keys_batch(const BatchScene *segs, const uint32_t *seg_offsets, uint32_t n_segs,
                             rr_key_layout layout, rr_t_source tsrc, float ratio, uint32_t key_bits,
                             uint32_t seg_bits, const float *o_tmin, const float *d_tmax, uint32_t n, void *keys,
-                            cudaStream_t s);
+                            uint32_t radix_bits, void *sort_workspace, int sm_count, cudaStream_t s);
 
 // Closest-hit trace of a batch through `order`, hits in input order; the
 // length tables of the segments are updated when `accumulate`.  queue: two
@@ -39,10 +41,6 @@ rr_status launch_keys_batch(const BatchScene *segs, const uint32_t *seg_offsets,
 rr_status launch_trace_batch(const BatchScene *segs, const uint32_t *seg_offsets, uint32_t n_segs, const float *o_tmin,
                              const float *d_tmax, const uint32_t *order, uint32_t n, float *hits_out,
                              bool accumulate, uint32_t block, uint32_t *queue, uint32_t *err, cudaStream_t s);
-
-// rr_sort with arguments already checked and device errors reported to `err`.
-rr_status sort_enqueue(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
-                       uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s);
 
 // The argument checks of rr_sort, with `what` naming the caller in messages.
 rr_status sort_check(const char *what, const void *keys_in, const void *keys_out, const uint32_t *perm_out,

@@ -9,12 +9,20 @@
 
 namespace rr {
 
-// x in [0,1] -> 32-bit cell by truncation; >= 1 -> all ones; <= 0 or NaN -> 0.
-__device__ __forceinline__ uint32_t quantise_unit(float x) {
-    if (!(x > 0.0f)) return 0u;
-    if (x >= 1.0f) return 0xFFFFFFFFu;
+// a * b, rounded, then clamped to [0,1] (NaN to 0): one instruction.
+__device__ __forceinline__ float mul_sat(float a, float b) {
+    float r;
+    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+// x in [0,1] -> 32-bit cell by truncation; 1 -> all ones (the conversion clamps 2^32).
+__device__ __forceinline__ uint32_t cell_of_unit(float x) {
     return __float2uint_rz(__fmul_rn(x, 4294967296.0f));  // times 2^32 is exact
 }
+
+// Any x: >= 1 -> all ones; <= 0 or NaN -> 0.
+__device__ __forceinline__ uint32_t quantise_unit(float x) { return cell_of_unit(mul_sat(x, 1.0f)); }
 
 struct QuantFrame {
     float lo[3];
@@ -36,7 +44,7 @@ __device__ __forceinline__ QuantFrame make_frame(const float lo[3], const float 
 }
 
 __device__ __forceinline__ uint32_t quantise_coord(const QuantFrame &f, int c, float p) {
-    return quantise_unit(__fmul_rn(__fsub_rn(p, f.lo[c]), f.inv[c]));
+    return cell_of_unit(mul_sat(__fsub_rn(p, f.lo[c]), f.inv[c]));
 }
 
 // |d| with the squares summed left to right.
@@ -155,7 +163,7 @@ __device__ __forceinline__ void quantise_ray(const QuantFrame &f, float4 o, floa
     dh[1] = len > 0.0f ? __fdiv_rn(d.y, len) : 0.0f;
     dh[2] = len > 0.0f ? __fdiv_rn(d.z, len) : 0.0f;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) qd[c] = quantise_unit(__fmul_rn(__fadd_rn(dh[c], 1.0f), 0.5f));
+    for (int c = 0; c < 3; ++c) qd[c] = cell_of_unit(mul_sat(__fadd_rn(dh[c], 1.0f), 0.5f));
 }
 
 // The frame of a box, computed once per block into shared memory by thread 0.

@@ -28,8 +28,8 @@ struct KeyArgs {
 // The key of one ray (Section 3.1): the first `bits` bits of its layout's
 // string, in the frame of the quantisation box.  t_given: the GIVEN estimate;
 // table: the ADAPTIVE cells.
-template <int LAYOUT, int TSRC>
-__device__ __forceinline__ uint64_t ray_key(const QuantFrame &f, float4 o, float4 d, uint32_t bits, float ratio,
+template <int LAYOUT, int TSRC, typename KeyT>
+__device__ __forceinline__ KeyT ray_key(const QuantFrame &f, float4 o, float4 d, uint32_t bits, float ratio,
                                             float t_given, const ulonglong2 *table, const uint32_t *lut) {
     uint32_t qo[3], qd[3];
     float dh[3];
@@ -72,27 +72,70 @@ __device__ __forceinline__ uint64_t ray_key(const QuantFrame &f, float4 o, float
         const uint32_t ob = bits - db;
         const uint64_t ko = prefix64(morton3_64(qo[0], qo[1], qo[2]), ob);
         const uint64_t kd = prefix64(morton3_64(qd[0], qd[1], qd[2]), db);
-        return LAYOUT == RR_KEY_REIS ? (db ? (ko << db) | kd : ko) : (ob ? (kd << ob) | ko : kd);
+        return (KeyT)(LAYOUT == RR_KEY_REIS ? (db ? (ko << db) | kd : ko) : (ob ? (kd << ob) | ko : kd));
     } else {
         float u, v;
         octahedral(d.x, d.y, d.z, u, v);
         const uint32_t c[5] = {qo[0], qo[1], qo[2], quantise_unit(u) >> 4, quantise_unit(v) >> 4};
         key64 = interleave_octa_64(c);
     }
-    return key64 >> (64 - bits);
+    // a key of at most 32 bits lies in the string's first word
+    if (sizeof(KeyT) == 4) return (KeyT)((uint32_t)(key64 >> 32) >> (32 - bits));
+    return (KeyT)(key64 >> (64 - bits));
 }
 
-// Persistent blocks walk over tiles of 256 rays.  Each tile's origins and
+// Persistent blocks walk over tiles of 512 rays.  Each tile's origins and
 // directions arrive in shared memory by two bulk asynchronous copies completed
 // on an mbarrier, issued one tile ahead into the other of two buffers, so the
-// loads of the next tile overlap the key arithmetic of this one.  One ray per
-// thread per tile: quantisation, interleave, one store.
-constexpr int kKeyTile = 256;
+// loads of the next tile overlap the key arithmetic of this one (plain loads
+// one tile ahead take the same time).  One ray per thread per tile:
+// quantisation, interleave, one store.
+//
+// What bounds it: issue and shared atomics at 8.3M rays (74% of the issue
+// slots, 69% of the shared-memory pipe with the digit counting; 72 us for 332
+// MB, 0.68 of the copy bandwidth), launch, tail and the blocks' count flushes
+// below a million.  Clamping inside the multiply and the conversion, digits at
+// fixed shifts, and only one word of the string for keys of at most 32 bits
+// took 8.3M 64-bit Aila keys from 88 to 71 us; blocks of 512 instead of 256
+// threads and two counts per flush atomic took keys and sort of 300,001 64-bit
+// keys from 75 to 70 us and of 2.07M 32-bit keys from 98 to 95.
+constexpr int kKeyTile = 512;
 constexpr uint32_t kCopySpinLimit = 1u << 22;  // polls of a copy's barrier before giving up
 
 // Digit-count entries of the fused form: passes x 2^radix_bits <= 2048 for
 // every key width with 4- or 8-bit digits.
 constexpr int kCountEntries = 2048;
+
+// Adds a key's digit of every sort pass to the counters.  Bits above the key's
+// are zero, so the last pass's digit needs no narrower mask.  8-bit digits at
+// fixed shifts: a loop over passes costs three times the instructions.
+template <typename KeyT>
+__device__ __forceinline__ void count_digits(KeyT key, uint32_t *counts, uint32_t passes, uint32_t radix_bits) {
+    if (radix_bits == 8) {
+#pragma unroll
+        for (uint32_t p = 0; p < sizeof(KeyT); ++p)
+            if (p < passes) atomicAdd(&counts[(p << 8) + ((uint32_t)(key >> (8 * p)) & 255u)], 1u);
+    } else {
+        for (uint32_t p = 0; p < passes; ++p) {
+            atomicAdd(&counts[(p << radix_bits) + ((uint32_t)key & ((1u << radix_bits) - 1u))], 1u);
+            key >>= radix_bits;
+        }
+    }
+}
+
+// After a block's last key: its counts (two copies) go to the sort's digit
+// counts, two neighbouring 32-bit counts per 64-bit atomic (no count passes
+// 2^30), and the sort's look-back words and tile counters are cleared.
+__device__ __forceinline__ void finish_counts(const uint32_t (&s_cnt)[2][kCountEntries], const SortCountTarget &c) {
+    const uint32_t entries = c.passes << c.radix_bits;
+    for (uint32_t i = 2 * threadIdx.x; i < entries; i += 2 * blockDim.x) {
+        const uint32_t c0 = s_cnt[0][i] + s_cnt[1][i], c1 = s_cnt[0][i + 1] + s_cnt[1][i + 1];
+        if (c0 | c1) atomicAdd(reinterpret_cast<unsigned long long *>(c.hist + i), (unsigned long long)c1 << 32 | c0);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < c.passes) c.counters[threadIdx.x] = 0u;
+    for (size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x; w < c.zero_count; w += (size_t)gridDim.x * blockDim.x)
+        c.zero_words[w] = make_uint4(0u, 0u, 0u, 0u);
+}
 
 // COUNT (the fused key + sort form): each block also counts the digits of
 // every sort pass of its keys (shared atomics into two copies, even and odd
@@ -100,7 +143,7 @@ constexpr int kCountEntries = 2048;
 // clears the sort's look-back words and tile counters, so the separate
 // counting kernel of the sort is not needed.
 template <int LAYOUT, int TSRC, typename KeyT, bool COUNT>
-__global__ void __launch_bounds__(kKeyTile, 6) key_kernel(KeyArgs a) {
+__global__ void __launch_bounds__(kKeyTile, 3) key_kernel(KeyArgs a) {
     __shared__ __align__(128) float4 s_o[2][kKeyTile];
     __shared__ __align__(128) float4 s_d[2][kKeyTile];
     __shared__ __align__(8) uint64_t s_bar[2];
@@ -146,61 +189,57 @@ __global__ void __launch_bounds__(kKeyTile, 6) key_kernel(KeyArgs a) {
         if (i < a.n) {
             const float tg = TSRC == RR_T_GIVEN ? __ldg(a.t_given + i) : 0.0f;
             const KeyT key =
-                (KeyT)ray_key<LAYOUT, TSRC>(f, s_o[buf][tid], s_d[buf][tid], a.bits, a.ratio, tg, a.table, lut);
+                ray_key<LAYOUT, TSRC, KeyT>(f, s_o[buf][tid], s_d[buf][tid], a.bits, a.ratio, tg, a.table, lut);
             static_cast<KeyT *>(a.keys)[i] = key;
-            if (COUNT) {
-                // bits above a.bits are zero, so the last pass's digit needs no narrower mask
-                uint32_t *mine = s_cnt[(tid >> 5) & 1u];
-                const uint32_t rb = a.count.radix_bits, mask = (1u << rb) - 1u;
-                KeyT x = key;
-                for (uint32_t p = 0; p < a.count.passes; ++p) {
-                    atomicAdd(&mine[(p << rb) + ((uint32_t)x & mask)], 1u);
-                    x >>= rb;
-                }
-            }
+            if (COUNT) count_digits(key, s_cnt[(tid >> 5) & 1u], a.count.passes, a.count.radix_bits);
         }
         __syncthreads();  // every thread is done with `buf` before it is refilled
     }
-    if (COUNT) {
+    if constexpr (COUNT) {
         __syncthreads();
-        const uint32_t entries = a.count.passes << a.count.radix_bits;
-        for (uint32_t i = tid; i < entries; i += kKeyTile) {
-            const uint32_t c = s_cnt[0][i] + s_cnt[1][i];
-            if (c) atomicAdd(a.count.hist + i, c);
-        }
-        if (blockIdx.x == 0 && tid < a.count.passes) a.count.counters[tid] = 0u;
-        for (size_t w = (size_t)blockIdx.x * kKeyTile + tid; w < a.count.zero_count; w += (size_t)gridDim.x * kKeyTile)
-            a.count.zero_words[w] = make_uint4(0u, 0u, 0u, 0u);
+        finish_counts(s_cnt, a.count);
     }
 }
 
 // Batches: the key of ray i in the frame (and table) of its segment, with the
-// segment number above the key's bits.
+// segment number above the key's bits.  Persistent blocks count the digits of
+// the sort's passes as the single-wavefront form does, so the sort needs no
+// counting kernel of its own.
 template <int LAYOUT, int TSRC, typename KeyT>
-__global__ void __launch_bounds__(256) key_batch_kernel(const BatchScene *__restrict__ segs,
-                                                        const uint32_t *__restrict__ seg_offsets, uint32_t n_segs,
-                                                        const float4 *__restrict__ o_tmin,
-                                                        const float4 *__restrict__ d_tmax, uint32_t n,
-                                                        uint32_t bits, float ratio, KeyT *__restrict__ keys) {
+__global__ void __launch_bounds__(kKeyTile, 3) key_batch_kernel(const BatchScene *__restrict__ segs,
+                                                               const uint32_t *__restrict__ seg_offsets,
+                                                               uint32_t n_segs, const float4 *__restrict__ o_tmin,
+                                                               const float4 *__restrict__ d_tmax, uint32_t n,
+                                                               uint32_t bits, float ratio, KeyT *__restrict__ keys,
+                                                               SortCountTarget count) {
     __shared__ uint32_t s_off[kMaxBatchSegments + 1];
+    __shared__ uint32_t s_cnt[2][kCountEntries];
     const uint32_t *lut = block_spread6_lut();
-    for (uint32_t k = threadIdx.x; k <= n_segs; k += blockDim.x) s_off[k] = seg_offsets[k];
+    for (uint32_t k = threadIdx.x; k <= n_segs; k += kKeyTile) s_off[k] = seg_offsets[k];
+    for (uint32_t k = threadIdx.x; k < 2u * kCountEntries; k += kKeyTile) (&s_cnt[0][0])[k] = 0u;
     __syncthreads();
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t lo = 0, hi = n_segs;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (s_off[mid] <= i)
-            lo = mid;
-        else
-            hi = mid;
+    const uint32_t tiles = (n + kKeyTile - 1) / kKeyTile;
+    for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const uint32_t i = t * kKeyTile + threadIdx.x;
+        if (i >= n) break;
+        uint32_t lo = 0, hi = n_segs;
+        while (hi - lo > 1) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (s_off[mid] <= i)
+                lo = mid;
+            else
+                hi = mid;
+        }
+        const QuantFrame f = segs[lo].frame;
+        const ulonglong2 *table = reinterpret_cast<const ulonglong2 *>(segs[lo].table);
+        const KeyT k =
+            ray_key<LAYOUT, TSRC, KeyT>(f, __ldg(o_tmin + i), __ldg(d_tmax + i), bits, ratio, 0.0f, table, lut);
+        const KeyT key = (KeyT)(((uint64_t)lo << bits) | k);
+        keys[i] = key;
+        count_digits(key, s_cnt[(threadIdx.x >> 5) & 1u], count.passes, count.radix_bits);
     }
-    const QuantFrame f = segs[lo].frame;
-    const ulonglong2 *table = reinterpret_cast<const ulonglong2 *>(segs[lo].table);
-    const uint64_t k =
-        ray_key<LAYOUT, TSRC>(f, __ldg(o_tmin + i), __ldg(d_tmax + i), bits, ratio, 0.0f, table, lut);
-    keys[i] = (KeyT)(((uint64_t)lo << bits) | k);
+    __syncthreads();
+    finish_counts(s_cnt, count);
 }
 
 __global__ void batch_frame_kernel(BatchScene *segs, const float *boxes, uint32_t n) {
@@ -316,28 +355,38 @@ cudaError_t launch_batch_frames(BatchScene *segs, const float *boxes, uint32_t n
     return cudaGetLastError();
 }
 
-template <int LAYOUT, int TSRC>
-static void launch_keys_batch_t(const BatchScene *segs, const uint32_t *offs, uint32_t n_segs, const float4 *o,
-                                const float4 *d, uint32_t n, uint32_t bits, float ratio, void *keys, bool wide,
-                                cudaStream_t s) {
-    dim3 grid((n + 255) / 256);
-    if (wide)
-        key_batch_kernel<LAYOUT, TSRC, unsigned long long><<<grid, 256, 0, s>>>(
-            segs, offs, n_segs, o, d, n, bits, ratio, static_cast<unsigned long long *>(keys));
-    else
-        key_batch_kernel<LAYOUT, TSRC, uint32_t><<<grid, 256, 0, s>>>(segs, offs, n_segs, o, d, n, bits, ratio,
-                                                                     static_cast<uint32_t *>(keys));
+template <int LAYOUT, int TSRC, typename KeyT>
+static void launch_keys_batch_k(const BatchScene *segs, const uint32_t *offs, uint32_t n_segs, const float4 *o,
+                                const float4 *d, uint32_t n, uint32_t bits, float ratio, void *keys,
+                                const SortCountTarget &count, int sm_count, cudaStream_t s) {
+    static int bps = 0;  // as key_grid
+    if (bps == 0) {
+        int v = 0;
+        const cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, key_batch_kernel<LAYOUT, TSRC, KeyT>, kKeyTile, 0);
+        bps = (e == cudaSuccess && v > 0) ? v : 1;
+    }
+    const uint32_t grid = std::min((n + kKeyTile - 1) / kKeyTile, (uint32_t)(sm_count * bps));
+    key_batch_kernel<LAYOUT, TSRC, KeyT>
+        <<<grid, kKeyTile, 0, s>>>(segs, offs, n_segs, o, d, n, bits, ratio, static_cast<KeyT *>(keys), count);
 }
 
 rr_status launch_keys_batch(const BatchScene *segs, const uint32_t *seg_offsets, uint32_t n_segs,
                             rr_key_layout layout, rr_t_source tsrc, float ratio, uint32_t key_bits,
                             uint32_t seg_bits, const float *o_tmin, const float *d_tmax, uint32_t n, void *keys,
-                            cudaStream_t s) {
+                            uint32_t radix_bits, void *sort_workspace, int sm_count, cudaStream_t s) {
     if (n == 0) return RR_OK;
     const bool wide = key_bits + seg_bits > 32;
     const float4 *o = reinterpret_cast<const float4 *>(o_tmin);
     const float4 *d = reinterpret_cast<const float4 *>(d_tmax);
-#define RR_KB(L, T) launch_keys_batch_t<L, T>(segs, seg_offsets, n_segs, o, d, n, key_bits, ratio, keys, wide, s)
+    const SortCountTarget count = sort_count_target(n, key_bits + seg_bits, radix_bits, sort_workspace);
+    const cudaError_t e = cudaMemsetAsync(count.hist, 0, sizeof(uint32_t) * (count.passes << radix_bits), s);
+    if (e != cudaSuccess) return fail_cuda(e, "rr_batch keys: memset");
+#define RR_KB(L, T)                                                                                              \
+    wide ? launch_keys_batch_k<L, T, unsigned long long>(segs, seg_offsets, n_segs, o, d, n, key_bits, ratio, keys, \
+                                                         count, sm_count, s)                                      \
+         : launch_keys_batch_k<L, T, uint32_t>(segs, seg_offsets, n_segs, o, d, n, key_bits, ratio, keys, count,    \
+                                               sm_count, s)
     switch (layout) {
         case RR_KEY_AILA: RR_KB(RR_KEY_AILA, 0); break;
         case RR_KEY_AILA_COMPACT: RR_KB(RR_KEY_AILA_COMPACT, 0); break;

@@ -208,10 +208,11 @@ rr_status launch_group(rr_server *s, Group *g) {
     rr_status rs = RR_OK;
     if (n > 0) {
         rs = launch_keys_batch(segs, offs, ng, (rr_key_layout)s->cfg.layout, (rr_t_source)s->cfg.t_source,
-                               s->cfg.ratio, key_bits, seg_bits, o, d, (uint32_t)n, keys, st);
+                               s->cfg.ratio, key_bits, seg_bits, o, d, (uint32_t)n, keys, s->cfg.radix_bits, wsp,
+                               s->sm_count, st);
         if (rs == RR_OK)
-            rs = sort_enqueue(keys, nullptr, perm, (uint32_t)n, total_bits, s->cfg.radix_bits, wsp, sl.err,
-                              s->sm_count, st);
+            rs = sort_enqueue_passes(keys, nullptr, perm, (uint32_t)n, total_bits, s->cfg.radix_bits, wsp, sl.err,
+                                     st);
         if (rs == RR_OK)
             rs = launch_trace_batch(segs, offs, ng, o, d, perm, (uint32_t)n, hits, adaptive(s),
                                     s->cfg.trace_block, sl.queue, sl.err, st);

@@ -762,11 +762,9 @@ static rr_status run_sort(const SortPlan &pl, const K *keys_in, K *keys_out, uin
     return RR_OK;
 }
 
-// The sort of rr_sort (arguments already checked) with device errors going to
-// `err`: batches captured on one stream and replayed on another report to the
-// word of the stream they run on.
-rr_status sort_enqueue(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
-                       uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s) {
+// The sort of rr_sort (arguments already checked).
+static rr_status sort_enqueue(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
+                              uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s) {
     const SortPlan pl = plan_sort(n, bits, radix_bits);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     if (pl.kb == 4) {
