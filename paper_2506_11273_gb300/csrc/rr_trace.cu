@@ -680,6 +680,132 @@ __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool li
     return more;
 }
 
+// One step of launches of few rays: up to four pending triangles and, unless
+// triangles of two groups are left after them, the next node, which is loaded
+// before the triangles are tested, so that both latencies overlap (80
+// registers: the tail of trace_kernel has no room for it, and the two steps
+// compiled from one source disturb its main loop).  Returns as quad_step.
+template <bool ANY, int BLOCK>
+__device__ __forceinline__ bool quad_step_early(RayState &r, RegisterExtra &x, bool live, uint2 *stack, const SceneRef &sc,
+                                           uint32_t *err, const uint8_t *s_oct) {
+    constexpr int L = 4, P = 8 / L;
+    constexpr uint32_t LANES = (1u << L) - 1u;
+    const uint32_t lane = threadIdx.x & 31u, quad = lane / L, j = lane % L;
+    // the triangles this step tests, and the node it visits
+    uint32_t left = r.t.hits, mine = left;
+#pragma unroll
+    for (uint32_t q = 0; q < (uint32_t)L; ++q) {
+        if (q == j) mine = left;
+        left &= left - 1u;
+    }
+    const bool test = live && r.t.hits != 0u;
+    bool visit = live && (r.u_hits == 0u || left == 0u);
+    if (visit && (r.g_mask & 0xFFu) == 0u) {
+        if (r.sp == 0) {
+            visit = false;
+        } else {
+            --r.sp;
+            const uint2 e = stack[quad_entry<BLOCK>(r.sp, quad)];
+            r.g_base = e.x;
+            r.g_mask = e.y;
+        }
+    }
+    const bool more = visit || test;
+    Words8 n0{}, n1{}, n2{};
+    uint32_t node = 0u;
+    if (visit) {
+        node = take_child(r);
+        visit = index_ok(node, sc.n_nodes, err);
+        if ((r.g_mask & 0xFFu) != 0u) {
+            if (r.sp < (int)kTraceStack) {
+                stack[quad_entry<BLOCK>(r.sp, quad)] = make_uint2(r.g_base, r.g_mask);  // its lanes store the same
+            } else {
+                atomicOr(err, RR_DEVERR_TRACE_STACK);
+                visit = false;
+            }
+            ++r.sp;
+        }
+        if (!visit) {
+            x.set_hit(0.0f, 0.0f, kMiss);
+            ray_stop(r);
+        } else {
+            const DevNode *np = sc.nodes + node;
+            n0 = load256(np);
+            n1 = load256(&np->qlo_x);
+            n2 = load256(&np->qlo_z);
+        }
+    }
+    if (__any_sync(0xFFFFFFFFu, test)) {
+        float u = 0.0f, v = 0.0f, t = __int_as_float(0x7f800000);
+        uint32_t k = kMiss;
+        bool hit = false;
+        if (live && r.t.hits != 0u) {
+            if (mine != 0u) {
+                k = r.t.base + __popc(r.t.all & ((mine & (0u - mine)) - 1u));
+                if (index_ok(k, sc.n_tris, err)) hit = meet_triangle(r, x.d(), sc, k, u, v, t);
+                if (!hit) t = __int_as_float(0x7f800000);
+            }
+            r.t.hits = left;
+            next_group(r, x);
+        }
+        const uint32_t hits = (__ballot_sync(0xFFFFFFFFu, hit) >> (L * quad)) & LANES;
+        if (__any_sync(0xFFFFFFFFu, hit)) {
+            // the winning lane: the nearest hit (ANY: the first), the first among equals
+            uint32_t win;
+            if (ANY) {
+                win = hits ? __ffs(hits) - 1u : 0u;
+            } else {
+                win = j;
+                float tw = t;
+#pragma unroll
+                for (int by = 1; by < L; by <<= 1) {
+                    const float to = __shfl_xor_sync(0xFFFFFFFFu, tw, by);
+                    const uint32_t wo = __shfl_xor_sync(0xFFFFFFFFu, win, by);
+                    if (to < tw || (to == tw && wo < win)) {
+                        tw = to;
+                        win = wo;
+                    }
+                }
+            }
+            const uint32_t from = L * quad + win;
+            const float tw = __shfl_sync(0xFFFFFFFFu, t, from), uw = __shfl_sync(0xFFFFFFFFu, u, from),
+                        vw = __shfl_sync(0xFFFFFFFFu, v, from);
+            const uint32_t kw = __shfl_sync(0xFFFFFFFFu, k, from);
+            if (hits != 0u) {
+                r.best = tw;
+                x.set_hit(uw, vw, kw);
+                if (ANY) {
+                    ray_stop(r);
+                    visit = false;
+                }
+            }
+        }
+    }
+    __syncwarp();
+    uint32_t in = 0u;  // bit i: slot j + L * i is hit
+    if (visit) {
+        const NodeSlabs s = node_slabs(r, n0, n1, n2);
+#pragma unroll
+        for (int i = 0; i < P; ++i) {
+            // byte of slot j + L * i, then the mantissa and exponent of 2^23
+            const uint32_t sel = 0x7540u | (j + (uint32_t)((L * i) & 3));
+            const int h = (L * i) / 4;
+            const auto at = [&](uint32_t w, float b, float a) {
+                return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), b, a);
+            };
+            const float t0 = max3f(at(s.nx[h], s.bx, s.ax), at(s.ny[h], s.by, s.ay), fmaxf(at(s.nz[h], s.bz, s.az), r.o.w));
+            const float t1 = min3f(at(s.fx[h], s.bx, s.ax), at(s.fy[h], s.by, s.ay), fminf(at(s.fz[h], s.bz, s.az), r.best));
+            if (t0 <= t1) in |= 1u << i;
+        }
+    }
+    uint32_t hm = 0u;
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+        hm |= ((__ballot_sync(0xFFFFFFFFu, (in >> i) & 1u) >> (L * quad)) & LANES) << (L * i);
+    if (visit) take_hits(r, x, n0, n2, hm, s_oct);
+    return more;
+}
+
 // Lanes refill from the queue once this many of a warp's 32 lanes are idle
 // (their rays finished): finished lanes write their hits together and idle
 // lanes take consecutive queue positions together.
@@ -888,7 +1014,7 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
 
 // Few rays: four lanes to a ray from the start.
 template <bool ACCUM, bool ANY, bool MULTI, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) trace_quad_kernel(TraceArgs a) {
+__global__ void __launch_bounds__(BLOCK, 768 / BLOCK) trace_quad_kernel(TraceArgs a) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ QuantFrame s_frame;
     __shared__ float s_invE;
@@ -921,7 +1047,7 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
             }
         }
         if (exhausted && __ballot_sync(0xFFFFFFFFu, live) == 0u) break;
-        const bool more = quad_step<ANY, BLOCK>(r, x, live, stack, cx.scene(seg), a.err, s_oct);
+        const bool more = quad_step_early<ANY, BLOCK>(r, x, live, stack, cx.scene(seg), a.err, s_oct);
         if (live && !more && (lane & 3u) == 0u) cx.store(r, x, ray, seg);
         live = more;
     }
@@ -1152,11 +1278,11 @@ extern "C" rr_status rr_bvh_aabb(const rr_bvh *b, float lo[3], float hi[3]) {
 
 namespace {
 
-// Launches of at most this many rays put four lanes to a ray: about as many as
-// the device then holds at once (152 SMs x 32 warps x 8).  A 4,097-ray bounce
-// takes 80 instead of 88 us; with 65,536 rays, two rounds of fours, it is
-// slower (172 against 148 us).
-constexpr uint32_t kQuadRays = 38912;
+// Launches of at most this many rays put four lanes to a ray (two lanes are
+// better than neither one nor four at any size).  Random order, one against four
+// lanes, us; tiny scene: 4,097 rays 50 / 40, 8,192 52 / 44, 16,384 53 / 51, 30,000
+// 57 / 63; 1,168,576 triangles: 16,384 92 / 83, 38,912 97 / 102.
+constexpr uint32_t kQuadRays = 16384;
 
 template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
 void *trace_entry() {

@@ -13,7 +13,7 @@ from paper_2506_11273_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
-N = 38912 + 4099  # above the largest launch that gets four lanes to a ray
+N = 38912 + 4099  # well above the largest launch that gets four lanes to a ray
 
 
 @pytest.fixture(scope="module")
@@ -33,7 +33,7 @@ def _trace(bvh, o, d, **kw):
 
 
 @pytest.mark.parametrize("flags", [0, rr.RR_TRACE_ANY_HIT])
-@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 31, 32, 33, 4097, 38911, 38912, 38913])
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 31, 32, 33, 4097, 16383, 16384, 16385, 38911, 38912, 38913])
 def test_small_launches_match_a_large_one(soup, n, flags):
     _, bvh, _, o, d = soup
     whole = _trace(bvh, o, d, flags=flags)
