@@ -108,6 +108,34 @@ constexpr bool kChecked = false;
 #endif
 
 #ifdef __CUDACC__
+// Programmatic dependent launch: a kernel lets the next kernel of its stream
+// start its blocks once all of its own have started, and waits (before it
+// touches global memory) until the kernel before it has finished and its
+// writes are visible.  Both are no-ops for a kernel launched without the
+// programmatic-serialisation attribute.
+__device__ __forceinline__ void allow_dependent_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_prerequisite() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launches a kernel with that attribute: launch and drain of neighbouring
+// kernels of a stream overlap.  The kernel calls wait_for_prerequisite().
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t s,
+                             const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 __device__ __forceinline__ bool index_ok(uint32_t i, uint32_t n, uint32_t *err) {
     if (!kChecked || i < n) return true;
     atomicOr(err, RR_DEVERR_BAD_INDEX);

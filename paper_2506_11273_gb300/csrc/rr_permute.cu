@@ -16,6 +16,8 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *__
                                                                float4 *__restrict__ o_out,
                                                                float4 *__restrict__ d_out,
                                                                uint32_t *__restrict__ p_out, uint32_t *err) {
+    allow_dependent_launch();
+    wait_for_prerequisite();
     const uint32_t base = blockIdx.x * (kPermuteBlock * kPermuteItems) + threadIdx.x;
     uint32_t src[kPermuteItems];
 #pragma unroll
@@ -84,6 +86,7 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_phased_kernel(
     const float4 *__restrict__ o_in, const float4 *__restrict__ d_in, const uint32_t *__restrict__ p_in,
     const uint32_t *__restrict__ perm, uint32_t n, float4 *__restrict__ o_out, float4 *__restrict__ d_out,
     uint32_t *__restrict__ p_out, uint32_t phase_blocks, uint32_t *err) {
+    wait_for_prerequisite();
     const uint32_t phase = blockIdx.x / phase_blocks, block = blockIdx.x - phase * phase_blocks;
     if (phase == 0)
         gather_phase(o_in, perm, n, o_out, block, err);
@@ -123,22 +126,20 @@ extern "C" rr_status rr_permute(const float *o_tmin_in, const float *d_tmax_in, 
     rr_status st;
     DeviceState *ds = device_state(&st);
     if (!ds) return st;
-    const uint32_t per_block = kPermuteBlock * kPermuteItems;
-    dim3 grid((n + per_block - 1) / per_block);
     cudaStream_t s = as_stream(stream);
     const float4 *oi = reinterpret_cast<const float4 *>(o_tmin_in);
     const float4 *di = reinterpret_cast<const float4 *>(d_tmax_in);
     float4 *oo = reinterpret_cast<float4 *>(o_tmin_out);
     float4 *dd = reinterpret_cast<float4 *>(d_tmax_out);
     uint32_t *err = error_word(ds, s);
+    const uint32_t blocks = (n + kPermuteBlock * kPermuteItems - 1) / (kPermuteBlock * kPermuteItems);
     if (n >= kPhasedRays) {
         const uint32_t phase_blocks = (n + kPermuteBlock * kPhaseItems - 1) / (kPermuteBlock * kPhaseItems);
-        permute_phased_kernel<<<phase_blocks * (payload_in ? 3u : 2u), kPermuteBlock, 0, s>>>(
-            oi, di, payload_in, perm, n, oo, dd, payload_out, phase_blocks, err);
-    } else if (payload_in) {
-        permute_kernel<true><<<grid, kPermuteBlock, 0, s>>>(oi, di, payload_in, perm, n, oo, dd, payload_out, err);
+        launch_dependent(permute_phased_kernel, phase_blocks * (payload_in ? 3u : 2u), kPermuteBlock, 0, s, oi, di,
+                         payload_in, perm, n, oo, dd, payload_out, phase_blocks, err);
     } else {
-        permute_kernel<false><<<grid, kPermuteBlock, 0, s>>>(oi, di, nullptr, perm, n, oo, dd, nullptr, err);
+        launch_dependent(payload_in ? permute_kernel<true> : permute_kernel<false>, blocks, kPermuteBlock, 0, s, oi, di,
+                         payload_in, perm, n, oo, dd, payload_out, err);
     }
     note_launches(1);
     return check_launch("rr_permute");

@@ -48,16 +48,6 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
-// Programmatic dependent launch: a pass lets the next kernel of its stream
-// start its blocks once all of its own have started, and waits (before it
-// touches global memory) until the kernel before it has finished and its
-// writes are visible.  Both are no-ops for a kernel launched without the
-// programmatic-serialisation attribute.
-__device__ __forceinline__ void allow_dependent_launch() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void wait_for_prerequisite() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Keys per thread of a full-size tile.
 template <typename K>
 struct SortTile {
@@ -622,17 +612,9 @@ constexpr size_t lookback_uint4(const SortPlan &p) { return (size_t)p.regions * 
 // drains (programmatic dependent launch; the pass waits in the kernel).
 template <typename K, int RBITS, int ITEMS, typename W, int MINB>
 static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((a.n + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS));
-    cfg.blockDim = dim3(kSortBlock);
-    cfg.dynamicSmemBytes = PassSmem<K, RBITS, ITEMS>::bytes;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, onesweep_kernel<K, RBITS, ITEMS, W, MINB>, a);
+    return launch_dependent(onesweep_kernel<K, RBITS, ITEMS, W, MINB>,
+                            (a.n + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS), kSortBlock,
+                            PassSmem<K, RBITS, ITEMS>::bytes, s, a);
 }
 
 // The pass in the plan's tile size (for 64-bit plans also the passes over the

@@ -292,29 +292,35 @@ __device__ __forceinline__ uint32_t take_child(RayState &r) {
     return r.g_base + __popc((r.g_mask >> 8) & ((1u << slot) - 1u));
 }
 
-// Hit masks of slot bits to octant positions (bit s to bit s ^ octant), a
-// table in shared memory: the three conditional swaps it replaces are a tenth
-// of the node visit's ALU work.
-struct OctantTable {
-    alignas(16) uint8_t at[8 * 256];
+// Tables of the node visit, in shared memory: hit masks from slot bits to octant
+// positions (bit s to bit s ^ octant), and leaf masks to the nibbles of their
+// slots.  The swaps and spreads they replace are ALU work, which the slab tests
+// already fill (2.07M camera rays 0.605 -> 0.586 ms).
+struct VisitTables {
+    alignas(16) uint8_t octant[8 * 256];
+    uint32_t nibbles[256];
 };
-constexpr OctantTable octant_table() {
-    OctantTable t{};
+constexpr VisitTables visit_tables() {
+    VisitTables t{};
     for (uint32_t k = 0; k < 8 * 256; ++k) {
         uint32_t h = k & 255u;
         if (k & 256u) h = ((h & 0x55u) << 1) | ((h >> 1) & 0x55u);
         if (k & 512u) h = ((h & 0x33u) << 2) | ((h >> 2) & 0x33u);
         if (k & 1024u) h = ((h & 0x0Fu) << 4) | (h >> 4);
-        t.at[k] = (uint8_t)h;
+        t.octant[k] = (uint8_t)h;
     }
+    for (uint32_t k = 0; k < 256; ++k)
+        for (uint32_t s = 0; s < 8; ++s)
+            if ((k >> s) & 1u) t.nibbles[k] |= 15u << (4 * s);
     return t;
 }
-__device__ const OctantTable g_octant_table = octant_table();
-__device__ __forceinline__ const uint8_t *block_octant_table() {
-    __shared__ OctantTable s_oct;
-    for (uint32_t k = threadIdx.x; k < 128u; k += blockDim.x)
-        reinterpret_cast<uint4 *>(s_oct.at)[k] = reinterpret_cast<const uint4 *>(g_octant_table.at)[k];
-    return s_oct.at;
+__device__ const VisitTables g_visit_tables = visit_tables();
+// Called by every thread; the caller synchronises the block afterwards.
+__device__ __forceinline__ const VisitTables &block_visit_tables() {
+    __shared__ VisitTables s_tables;
+    for (uint32_t k = threadIdx.x; k < sizeof(VisitTables) / 16; k += blockDim.x)
+        reinterpret_cast<uint4 *>(&s_tables)[k] = reinterpret_cast<const uint4 *>(&g_visit_tables)[k];
+    return s_tables;
 }
 
 __device__ __forceinline__ float max3f(float a, float b, float c) {
@@ -380,16 +386,12 @@ __device__ __forceinline__ NodeSlabs node_slabs(const RayState &r, const Words8 
 // children) and its last pending triangle group (leaves).
 template <typename X>
 __device__ __forceinline__ void take_hits(RayState &r, X &x, const Words8 &n0, const Words8 &n2, uint32_t hm,
-                                          const uint8_t *s_oct) {
+                                          const VisitTables &tables) {
     const uint32_t imask = n0.w[3] & 0xFFu, tribits = n2.w[5];
     hm &= n0.w[3] >> 8;  // used slots only
-    const uint32_t hits = s_oct[r.negmask * 256u + (hm & imask)];
+    const uint32_t hits = tables.octant[r.negmask * 256u + (hm & imask)];
     // leaves: slot bit s -> nibble s, keeping the triangles the nibble holds
-    uint32_t leaf = hm & ~imask;
-    leaf = (leaf | (leaf << 12)) & 0x000F000Fu;
-    leaf = (leaf | (leaf << 6)) & 0x03030303u;
-    leaf = (leaf | (leaf << 3)) & 0x11111111u;
-    const uint32_t tris = (leaf * 15u) & tribits;
+    const uint32_t tris = tables.nibbles[hm & ~imask] & tribits;
     r.g_base = n0.w[7];
     r.g_mask = hits | (imask << 8);
     if (tris != 0u) {
@@ -506,7 +508,7 @@ __device__ __forceinline__ void accumulate_hit(unsigned long long *table, const 
 // that would overflow records RR_DEVERR_TRACE_STACK and ends the ray as a miss.
 template <bool ANY, bool LEAN, int BLOCK>
 __device__ __forceinline__ bool ray_step(RayState &r, LaneExtra<LEAN, BLOCK> &x, bool live, uint2 *l_stack,
-                                         const SceneRef &sc, uint32_t *err, const uint8_t *s_oct) {
+                                         const SceneRef &sc, uint32_t *err, const VisitTables &tables) {
     uint2 *s_stack = x.m.stack + x.at;  // entries BLOCK apart
     bool more = live;
     if (live && r.t.hits != 0u) {
@@ -544,7 +546,7 @@ __device__ __forceinline__ bool ray_step(RayState &r, LaneExtra<LEAN, BLOCK> &x,
         if (ok) {
             const DevNode *np = sc.nodes + node;
             const Words8 n0 = load256(np), n1 = load256(&np->qlo_x), n2 = load256(&np->qlo_z);
-            take_hits(r, x, n0, n2, hit_slots(r, node_slabs(r, n0, n1, n2)), s_oct);
+            take_hits(r, x, n0, n2, hit_slots(r, node_slabs(r, n0, n1, n2)), tables);
         } else {
             x.set_hit(0.0f, 0.0f, kMiss);
             ray_stop(r);
@@ -577,7 +579,7 @@ __device__ __forceinline__ uint32_t quad_entry(uint32_t sp, uint32_t quad) {
 // for the lanes of a ray that is finished (or of no ray).
 template <bool ANY, int BLOCK>
 __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool live, uint2 *stack, const SceneRef &sc,
-                                          uint32_t *err, const uint8_t *s_oct) {
+                                          uint32_t *err, const VisitTables &tables) {
     const uint32_t lane = threadIdx.x & 31u, quad = lane >> 2, j = lane & 3u;
     const bool test = live && r.t.hits != 0u;
     if (__any_sync(0xFFFFFFFFu, test)) {
@@ -676,7 +678,7 @@ __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool li
         }
     }
     const uint32_t lo = __ballot_sync(0xFFFFFFFFu, two[0]), hi = __ballot_sync(0xFFFFFFFFu, two[1]);
-    if (visit) take_hits(r, x, n0, n2, ((lo >> (4u * quad)) & 15u) | (((hi >> (4u * quad)) & 15u) << 4), s_oct);
+    if (visit) take_hits(r, x, n0, n2, ((lo >> (4u * quad)) & 15u) | (((hi >> (4u * quad)) & 15u) << 4), tables);
     return more;
 }
 
@@ -687,7 +689,7 @@ __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool li
 // compiled from one source disturb its main loop).  Returns as quad_step.
 template <bool ANY, int BLOCK>
 __device__ __forceinline__ bool quad_step_early(RayState &r, RegisterExtra &x, bool live, uint2 *stack, const SceneRef &sc,
-                                           uint32_t *err, const uint8_t *s_oct) {
+                                           uint32_t *err, const VisitTables &tables) {
     constexpr int L = 4, P = 8 / L;
     constexpr uint32_t LANES = (1u << L) - 1u;
     const uint32_t lane = threadIdx.x & 31u, quad = lane / L, j = lane % L;
@@ -802,7 +804,7 @@ __device__ __forceinline__ bool quad_step_early(RayState &r, RegisterExtra &x, b
 #pragma unroll
     for (int i = 0; i < P; ++i)
         hm |= ((__ballot_sync(0xFFFFFFFFu, (in >> i) & 1u) >> (L * quad)) & LANES) << (L * i);
-    if (visit) take_hits(r, x, n0, n2, hm, s_oct);
+    if (visit) take_hits(r, x, n0, n2, hm, tables);
     return more;
 }
 
@@ -930,8 +932,10 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
     SceneRef *s_sc = reinterpret_cast<SceneRef *>(s_dyn);
     const TraceContext<ACCUM, MULTI> cx{a, s_sc, reinterpret_cast<uint32_t *>(s_sc + (MULTI ? a.n_segs : 0)), &s_frame,
                                         &s_invE};
+    allow_dependent_launch();
+    const VisitTables &tables = block_visit_tables();
+    wait_for_prerequisite();
     cx.load();
-    const uint8_t *s_oct = block_octant_table();
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t lanes_below = (1u << lane) - 1u;
@@ -961,7 +965,7 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
             }
             if (exhausted && (uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, live)) <= kTailRays) break;
         }
-        const bool more = ray_step<ANY, LEAN, BLOCK>(r, x, live, l_stack, cx.scene(seg), a.err, s_oct);
+        const bool more = ray_step<ANY, LEAN, BLOCK>(r, x, live, l_stack, cx.scene(seg), a.err, tables);
         finished = finished || (live && !more);
         live = more;
     }
@@ -1004,7 +1008,7 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
         }
         bool qlive = left != 0u;
         while (__any_sync(0xFFFFFFFFu, qlive)) {
-            const bool more = quad_step<ANY, BLOCK>(q, qx, qlive, stack, cx.scene(qseg), a.err, s_oct);
+            const bool more = quad_step<ANY, BLOCK>(q, qx, qlive, stack, cx.scene(qseg), a.err, tables);
             if (qlive && !more && (lane & 3u) == 0u) cx.store(q, qx, qray, qseg);
             qlive = more;
         }
@@ -1022,8 +1026,10 @@ __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) trace_quad_kernel(TraceArg
     SceneRef *s_sc = reinterpret_cast<SceneRef *>(s_dyn);
     const TraceContext<ACCUM, MULTI> cx{a, s_sc, reinterpret_cast<uint32_t *>(s_sc + (MULTI ? a.n_segs : 0)), &s_frame,
                                         &s_invE};
+    allow_dependent_launch();
+    const VisitTables &tables = block_visit_tables();
+    wait_for_prerequisite();
     cx.load();
-    const uint8_t *s_oct = block_octant_table();
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u, quad = lane >> 2;
     uint2 *stack = s_stack + (threadIdx.x & ~31u);
@@ -1047,7 +1053,7 @@ __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) trace_quad_kernel(TraceArg
             }
         }
         if (exhausted && __ballot_sync(0xFFFFFFFFu, live) == 0u) break;
-        const bool more = quad_step_early<ANY, BLOCK>(r, x, live, stack, cx.scene(seg), a.err, s_oct);
+        const bool more = quad_step_early<ANY, BLOCK>(r, x, live, stack, cx.scene(seg), a.err, tables);
         if (live && !more && (lane & 3u) == 0u) cx.store(r, x, ray, seg);
         live = more;
     }
@@ -1312,10 +1318,8 @@ void trace_enqueue_form(const TraceArgs &a, int sm_count, cudaStream_t s) {
     if (MULTI)  // static and dynamic shared memory together may pass the default 48 KB
         cudaFuncSetAttribute(trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)multi_smem(kMaxBatchSegments));
-    if (QUAD)
-        trace_quad_kernel<ACC, ANY, MULTI, BLOCK><<<grid, BLOCK, smem, s>>>(a);
-    else
-        trace_kernel<ACC, ANY, MULTI, BLOCK><<<grid, BLOCK, smem, s>>>(a);
+    launch_dependent(QUAD ? trace_quad_kernel<ACC, ANY, MULTI, BLOCK> : trace_kernel<ACC, ANY, MULTI, BLOCK>, grid, BLOCK,
+                     smem, s, a);
 }
 
 template <bool ACC, bool ANY, bool MULTI, int BLOCK>
