@@ -289,11 +289,15 @@ __global__ void table_init_kernel(ulonglong2 *cells) {
 }
 
 // After a trace: rays that hit add their fixed-point length to their cell.
-// Lanes of a warp that share a cell combine first (match_any + warp reduce),
-// then one lane issues the two 64-bit atomics.  Persistent blocks: the frame
-// (divisions, a barrier) is computed once for all the rays of a block.
+// Neighbouring lanes of a warp that share a cell combine first (a segmented
+// scan over runs of equal cells, which sorted rays have), then a run's last lane
+// issues the two 64-bit atomics.  What bounds it: the atomics (1.2M rays: 57 MB
+// in 20 us).  Grouping all lanes of a cell by match and reduce costs a round per
+// distinct cell of the warp: 1.2M sorted rays 29.6 us against 19.8, in pixel
+// order 44 against 22, in random order 47 against 23.  Persistent blocks: the
+// frame (divisions, a barrier) is computed once for all the rays of a block.
 constexpr int kAccumulateBlock = 256;
-constexpr uint32_t kAccumulateBlocksPerSm = 8;  // 3 blocks: the 1.2M-ray bounce 652 -> 661 us; 5: the same
+constexpr uint32_t kAccumulateBlocksPerSm = 8;
 __global__ void __launch_bounds__(kAccumulateBlock) table_accumulate_kernel(unsigned long long *cells, Box box,
                                                                             const float4 *__restrict__ o_tmin,
                                                                             const float4 *__restrict__ d_tmax,
@@ -323,16 +327,24 @@ __global__ void __launch_bounds__(kAccumulateBlock) table_accumulate_kernel(unsi
                 valid = true;
             }
         }
-        const uint32_t vmask = __ballot_sync(0xFFFFFFFFu, valid);
-        if (valid) {
-            const uint32_t peers = __match_any_sync(vmask, cell);
-            const uint32_t s_hi = __reduce_add_sync(peers, lq >> 16);
-            const uint32_t s_lo = __reduce_add_sync(peers, lq & 0xFFFFu);
-            if (lane == (uint32_t)(__ffs(peers) - 1)) {
-                const unsigned long long sum = ((unsigned long long)s_hi << 16) + s_lo;
-                atomicAdd(cells + 2 * (size_t)cell, sum);
-                atomicAdd(cells + 2 * (size_t)cell + 1, (unsigned long long)__popc(peers));
+        // lq below 2^31 as two halves; the count above the high halves' sum
+        const uint32_t mine = valid ? cell : 0xFFFFFFFFu;
+        const uint32_t before = __shfl_up_sync(0xFFFFFFFFu, mine, 1);
+        const uint32_t heads = __ballot_sync(0xFFFFFFFFu, lane == 0u || before != mine);
+        const uint32_t start = 31u - __clz(heads & (0xFFFFFFFFu >> (31u - lane)));
+        uint32_t hi = (lq >> 16) | (1u << 24), lo = lq & 0xFFFFu;
+#pragma unroll
+        for (uint32_t by = 1; by < 32; by <<= 1) {
+            const uint32_t h2 = __shfl_up_sync(0xFFFFFFFFu, hi, by), l2 = __shfl_up_sync(0xFFFFFFFFu, lo, by);
+            if (lane >= start + by) {
+                hi += h2;
+                lo += l2;
             }
+        }
+        const bool last = lane == 31u || ((heads >> (lane + 1u)) & 1u);
+        if (valid && last) {
+            atomicAdd(cells + 2 * (size_t)cell, ((unsigned long long)(hi & 0xFFFFFFu) << 16) + lo);
+            atomicAdd(cells + 2 * (size_t)cell + 1, (unsigned long long)(hi >> 24));
         }
         __syncwarp();
     }
