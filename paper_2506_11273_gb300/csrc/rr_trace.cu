@@ -90,6 +90,17 @@ __device__ __forceinline__ Words8 load256(const void *p) {
     return r;
 }
 
+// A ray is read once: its loads and its hit's store leave L1 to the BVH (2.07M
+// camera rays 0.583 -> 0.578 ms, 8.3M random-order rays 2.79 -> 2.77; triangles
+// loaded the same way lose 3% on scenes whose triangles L1 holds).
+__device__ __forceinline__ float4 load_once(const float4 *p) {
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+        : "l"(p));
+    return v;
+}
+
 // Error-free transformations (Knuth's TwoSum, FMA-based TwoProd).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);
@@ -893,7 +904,7 @@ struct TraceContext {
     template <typename X>
     __device__ __forceinline__ void store(const RayState &r, const X &x, uint32_t ray, uint32_t seg) const {
         const float4 h = ray_result(r, x, scene(seg));
-        a.hits[ray] = h;
+        __stcs(a.hits + ray, h);
         if (ACCUM) {
             if (MULTI) {
                 const BatchScene *bs = a.segs + seg;
@@ -959,7 +970,7 @@ __global__ void __launch_bounds__(BLOCK, (trace_min_blocks<MULTI, BLOCK>())) tra
                 base = __shfl_sync(0xFFFFFFFFu, base, 0);
                 if (base + want >= a.n) exhausted = true;
                 if (!live && cx.find_ray(base + __popc(idle & lanes_below), ray, seg)) {
-                    ray_begin(r, x, cx.scene(seg), __ldg(a.o_tmin + ray), __ldg(a.d_tmax + ray));
+                    ray_begin(r, x, cx.scene(seg), load_once(a.o_tmin + ray), load_once(a.d_tmax + ray));
                     live = true;
                 }
             }
@@ -1048,7 +1059,7 @@ __global__ void __launch_bounds__(BLOCK, 768 / BLOCK) trace_quad_kernel(TraceArg
             base = __shfl_sync(0xFFFFFFFFu, base, 0);
             if (base + want >= a.n) exhausted = true;
             if (!live && cx.find_ray(base + ((uint32_t)__popc(idle & ((1u << (4u * quad)) - 1u)) >> 2), ray, seg)) {
-                ray_begin(r, x, cx.scene(seg), __ldg(a.o_tmin + ray), __ldg(a.d_tmax + ray));
+                ray_begin(r, x, cx.scene(seg), load_once(a.o_tmin + ray), load_once(a.d_tmax + ray));
                 live = true;
             }
         }
