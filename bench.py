@@ -49,7 +49,7 @@ TRACE_SOURCES = ["paper_2506_11273_gb300/csrc/rr_trace.cu", "paper_2506_11273_gb
 # rays, `trace_kernel<0, 0, 0, 128>`): DRAM bytes read + written and warp
 # instructions per launch, valid only while the trace sources hash to `sources`
 # (sha256 of TRACE_SOURCES, first 16 hex digits); otherwise traffic is reported as null.
-TRACE_NCU = {"sources": "16c2fbc1e738e3cd", "dram_bytes": 171183616 + 16250624, "warp_instructions": 540485561}
+TRACE_NCU = {"sources": "5adfdf8d3c13586f", "dram_bytes": 132669696 + 12462080, "warp_instructions": 376998630}
 # issue-slot peak: 4 warp instructions per cycle per SM (one per scheduler) x 152 SMs
 SMS, ISSUE_PER_SM_CYCLE, MAX_SM_MHZ = 152, 4, 2070.0
 

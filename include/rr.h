@@ -124,8 +124,8 @@ typedef struct {
     uint32_t n_nodes;  /* 8-wide nodes */
     uint32_t n_leaves; /* leaf slots (1..4 triangles each) */
     uint32_t depth;    /* node levels from the root to the deepest node */
-    uint64_t node_bytes;
-    uint64_t tri_bytes;
+    uint64_t node_bytes; /* of the nodes in the serialized form */
+    uint64_t tri_bytes;  /* of the triangles and their planes in the serialized form */
     float aabb_lo[3];
     float aabb_hi[3];
     double build_seconds;

@@ -269,9 +269,9 @@ extern "C" rr_status rr_pipeline_run_host(rr_pipeline *p, const float *o_host, c
     uint64_t ticket = 0;
     // A caller that waits for this bounce has nothing to overlap the hits' way
     // back with but the trace itself, so into page-locked hits the trace stores
-    // directly (wall time of the call: 1.2M rays 0.89 -> 0.79 ms).  Not with the length-table update,
-    // which reads the hits again, and not for streams of submissions, whose
-    // copies overlap the next bounce.
+    // directly (the whole call: 1.2M rays 0.89 -> 0.79 ms).  Not with the
+    // length-table update, which reads the hits again, and not for streams of
+    // submissions, whose copies overlap the next bounce.
     float *direct = nullptr;
     if (p && n > 0 && n <= p->max_n && !bounce_updates_table(p) && aligned16(hits_host))
         direct = static_cast<float *>(mapped_host_range(hits_host, 16ull * n));

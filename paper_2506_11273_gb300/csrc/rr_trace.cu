@@ -20,8 +20,8 @@
 // memory, and a warp whose last rays run on hands each to four lanes.
 // Measured against the earlier form (one step a triangle or a node, 128-bit
 // loads of 80-byte nodes, local stack), 1,168,576 triangles: 2.07M camera rays
-// 0.723 -> 0.582 ms, 8.3M random-order secondary rays 3.38 -> 2.78 ms, 0.99M
-// any-hit shadow rays 0.273 -> 0.235 ms.
+// 0.722 -> 0.574 ms, 8.3M random-order secondary rays 3.39 -> 2.77 ms, 0.99M
+// any-hit shadow rays 0.273 -> 0.230 ms.
 //
 // Two variants serve the reordering study: indirect access (the queue hands
 // out positions of an index buffer, so sorted rays are traced without being
