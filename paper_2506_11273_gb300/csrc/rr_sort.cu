@@ -388,9 +388,8 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
 }
 
 // MINB blocks per SM: 3 for passes of one wave or less (shortest tile
-// latency), 4 with late values for longer passes (more tiles in flight: 506
-// tiles of 2.07M 32-bit keys, which three blocks per SM would run as one full
-// and one nearly empty wave, 105 -> 99 us for keys and sort).
+// latency), 4 for longer passes (more tiles in flight).  Passes of four blocks
+// and of tiles above the full size load the values late.
 template <typename K, int RBITS, int ITEMS, typename W, int MINB>
 __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> a) {
     using L = PassSmem<K, RBITS, ITEMS>;
@@ -406,9 +405,9 @@ __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> 
     __syncthreads();
     const uint32_t tile = s_misc[0];
     if ((tile + 1) * (uint32_t)L::TILE <= a.n)
-        onesweep_tile<K, RBITS, ITEMS, W, true, (MINB > 3)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, true, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
     else
-        onesweep_tile<K, RBITS, ITEMS, W, false, (MINB > 3)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, false, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
 }
 
 // ------------------------------------------------------------------ local (segment) sort
@@ -549,8 +548,8 @@ struct SortPlan {
     size_t off_hist, off_counters, off_lookback, off_keys_a, off_keys_b, off_vals, total;
 };
 
-// Tiles of a pass that fit on the device at three blocks per SM (152 SMs).
-constexpr uint32_t kWaveTiles = 456;
+// Tiles of a pass that fit on the device at three and four blocks per SM (152 SMs).
+constexpr uint32_t kWaveTiles = 456, kWaveTiles4 = 608;
 
 constexpr uint32_t full_items(uint32_t kb) {
     return kb == 8 ? SortTile<unsigned long long>::kItems : SortTile<uint32_t>::kItems;
@@ -612,6 +611,12 @@ constexpr size_t lookback_uint4(const SortPlan &p) { return (size_t)p.regions * 
 // drains (programmatic dependent launch; the pass waits in the kernel).
 template <typename K, int RBITS, int ITEMS, typename W, int MINB>
 static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
+    if (PassSmem<K, RBITS, ITEMS>::bytes > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(onesweep_kernel<K, RBITS, ITEMS, W, MINB>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)PassSmem<K, RBITS, ITEMS>::bytes);
+        if (e != cudaSuccess) return e;
+    }
     return launch_dependent(onesweep_kernel<K, RBITS, ITEMS, W, MINB>,
                             (a.n + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS), kSortBlock,
                             PassSmem<K, RBITS, ITEMS>::bytes, s, a);
@@ -619,7 +624,13 @@ static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
 
 // The pass in the plan's tile size (for 64-bit plans also the passes over the
 // 32-bit high halves).  Full-size passes of more than one wave take the
-// four-block form.
+// four-block form, unless larger tiles keep the pass to one wave: 20 keys at
+// three blocks for 32-bit keys (1.87M to 2.33M keys; keys and sort of 1.9M 92.4
+// -> 86.4 us, 2.07M 95.3 -> 90.9, 2.3M 97.9 -> 92.0, but 2.6M 115.6 -> 118.3), 14
+// keys at four blocks for 64-bit keys (1.87M to 2.18M; with the 32-bit passes
+// over their high halves 1.9M 182 -> 174 us, 2.07M 194 -> 176, but 1.7M 149 -> 162
+// and 2.3M 201 -> 207).  No pass has more tiles than the one before it, which
+// clears its look-back words.
 template <typename K, int RBITS>
 static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaStream_t s) {
     using W64 = unsigned long long;
@@ -629,6 +640,12 @@ static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaS
     if (tiles12 <= kWaveTiles && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
     constexpr int FULL = SortTile<K>::kItems;
     const uint32_t tiles = (a.n + kSortBlock * FULL - 1) / (kSortBlock * FULL);
+    if constexpr (RBITS == 8) {  // (4-bit digits: not measured)
+        constexpr int LARGE = sizeof(K) == 8 ? 14 : 20;
+        constexpr uint32_t kWave = sizeof(K) == 8 ? kWaveTiles4 : kWaveTiles;
+        if (tiles > kWave && (a.n + kSortBlock * LARGE - 1) / (kSortBlock * LARGE) <= kWave)
+            return launch_pass<K, RBITS, LARGE, W64, sizeof(K) == 8 ? 4 : 3>(a, s);
+    }
     if (tiles > kWaveTiles) return launch_pass<K, RBITS, FULL, W64, 4>(a, s);
     return launch_pass<K, RBITS, FULL, W64, 3>(a, s);
 }
