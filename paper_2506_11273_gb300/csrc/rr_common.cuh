@@ -113,6 +113,12 @@ constexpr bool kChecked = false;
 // touches global memory) until the kernel before it has finished and its
 // writes are visible.  Both are no-ops for a kernel launched without the
 // programmatic-serialisation attribute.
+//
+// A kernel that waits is resident while the kernels before it still write, so
+// whatever an earlier kernel may have produced is read by ordinary loads after
+// the wait.  The read-only path (__ldg, ld.global.nc, const __restrict__
+// parameters) is for data that stays unchanged for the whole life of the reading
+// kernel, its time before the wait included: here only the BVH.
 __device__ __forceinline__ void allow_dependent_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

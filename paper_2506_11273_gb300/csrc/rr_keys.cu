@@ -299,10 +299,8 @@ __global__ void table_init_kernel(ulonglong2 *cells) {
 constexpr int kAccumulateBlock = 256;
 constexpr uint32_t kAccumulateBlocksPerSm = 8;
 __global__ void __launch_bounds__(kAccumulateBlock) table_accumulate_kernel(unsigned long long *cells, Box box,
-                                                                            const float4 *__restrict__ o_tmin,
-                                                                            const float4 *__restrict__ d_tmax,
-                                                                            const float4 *__restrict__ hits,
-                                                                            uint32_t n) {
+                                                                            const float4 *o_tmin, const float4 *d_tmax,
+                                                                            const float4 *hits, uint32_t n) {
     const QuantFrame f = block_frame(box.lo, box.hi);
     const float invE = __fdiv_rn(1.0f, f.E);
     wait_for_prerequisite();
@@ -313,7 +311,7 @@ __global__ void __launch_bounds__(kAccumulateBlock) table_accumulate_kernel(unsi
         bool valid = false;
         uint32_t cell = 0, lq = 0;
         if (i < n) {
-            const float4 h = __ldg(hits + i), o = __ldg(o_tmin + i), d = __ldg(d_tmax + i);
+            const float4 h = hits[i], o = o_tmin[i], d = d_tmax[i];
             if (__float_as_uint(h.w) != kMiss && isfinite(h.x)) {
                 uint32_t qo[3], qd[3];
                 float dh[3];

@@ -9,13 +9,10 @@ constexpr int kPermuteBlock = 256;
 constexpr int kPermuteItems = 2;  // rays per thread: more loads in flight per thread
 
 template <bool PAYLOAD>
-__global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *__restrict__ o_in,
-                                                               const float4 *__restrict__ d_in,
-                                                               const uint32_t *__restrict__ p_in,
-                                                               const uint32_t *__restrict__ perm, uint32_t n,
-                                                               float4 *__restrict__ o_out,
-                                                               float4 *__restrict__ d_out,
-                                                               uint32_t *__restrict__ p_out, uint32_t *err) {
+__global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *o_in, const float4 *d_in,
+                                                               const uint32_t *p_in, const uint32_t *perm,
+                                                               uint32_t n, float4 *o_out, float4 *d_out,
+                                                               uint32_t *p_out, uint32_t *err) {
     allow_dependent_launch();
     wait_for_prerequisite();
     const uint32_t base = blockIdx.x * (kPermuteBlock * kPermuteItems) + threadIdx.x;
@@ -31,9 +28,9 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *__
     for (int j = 0; j < kPermuteItems; ++j) {
         const uint32_t i = base + j * kPermuteBlock;
         if (i < n && index_ok(src[j], n, err)) {
-            o[j] = __ldg(o_in + src[j]);
-            d[j] = __ldg(d_in + src[j]);
-            if (PAYLOAD) p[j] = __ldg(p_in + src[j]);
+            o[j] = o_in[src[j]];
+            d[j] = d_in[src[j]];
+            if (PAYLOAD) p[j] = p_in[src[j]];
         }
     }
 #pragma unroll
@@ -60,8 +57,8 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *__
 constexpr int kPhaseItems = 4;  // rays per thread and array
 
 template <typename T>
-__device__ __forceinline__ void gather_phase(const T *__restrict__ in, const uint32_t *__restrict__ perm, uint32_t n,
-                                             T *__restrict__ out, uint32_t block, uint32_t *err) {
+__device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, uint32_t n, T *out,
+                                             uint32_t block, uint32_t *err) {
     const uint32_t base = block * (kPermuteBlock * kPhaseItems) + threadIdx.x;
     uint32_t src[kPhaseItems];
     T v[kPhaseItems];
@@ -73,7 +70,7 @@ __device__ __forceinline__ void gather_phase(const T *__restrict__ in, const uin
 #pragma unroll
     for (int j = 0; j < kPhaseItems; ++j) {
         const uint32_t i = base + j * kPermuteBlock;
-        if (i < n && index_ok(src[j], n, err)) v[j] = __ldg(in + src[j]);
+        if (i < n && index_ok(src[j], n, err)) v[j] = in[src[j]];
     }
 #pragma unroll
     for (int j = 0; j < kPhaseItems; ++j) {
@@ -83,9 +80,8 @@ __device__ __forceinline__ void gather_phase(const T *__restrict__ in, const uin
 }
 
 __global__ void __launch_bounds__(kPermuteBlock) permute_phased_kernel(
-    const float4 *__restrict__ o_in, const float4 *__restrict__ d_in, const uint32_t *__restrict__ p_in,
-    const uint32_t *__restrict__ perm, uint32_t n, float4 *__restrict__ o_out, float4 *__restrict__ d_out,
-    uint32_t *__restrict__ p_out, uint32_t phase_blocks, uint32_t *err) {
+    const float4 *o_in, const float4 *d_in, const uint32_t *p_in, const uint32_t *perm, uint32_t n, float4 *o_out,
+    float4 *d_out, uint32_t *p_out, uint32_t phase_blocks, uint32_t *err) {
     wait_for_prerequisite();
     const uint32_t phase = blockIdx.x / phase_blocks, block = blockIdx.x - phase * phase_blocks;
     if (phase == 0)

@@ -92,12 +92,14 @@ __device__ __forceinline__ Words8 load256(const void *p) {
 
 // A ray is read once: its loads and its hit's store leave L1 to the BVH (2.07M
 // camera rays 0.583 -> 0.578 ms, 8.3M random-order rays 2.79 -> 2.77; triangles
-// loaded the same way lose 3% on scenes whose triangles L1 holds).
+// loaded the same way lose 3% on scenes whose triangles L1 holds).  An ordinary
+// load behind the kernel's wait: the kernel before may have written the rays.
 __device__ __forceinline__ float4 load_once(const float4 *p) {
     float4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-        : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
     return v;
 }
 
@@ -879,7 +881,7 @@ struct TraceContext {
     // index buffer that is no permutation) no ray of the launch.
     __device__ __forceinline__ bool find_ray(uint32_t pos, uint32_t &ray, uint32_t &seg) const {
         if (pos >= a.n) return false;
-        const uint32_t i = a.order ? __ldg(a.order + pos) : pos;
+        const uint32_t i = a.order ? a.order[pos] : pos;
         if (i >= a.n) {  // not a permutation of [0, n): record and skip
             atomicOr(a.err, RR_DEVERR_BAD_INDEX);
             return false;
