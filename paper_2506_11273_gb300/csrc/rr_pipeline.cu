@@ -29,6 +29,7 @@ struct rr_pipeline {
     float *o_sorted, *d_sorted;
     HostSlot slot[2];
     cudaStream_t upload = nullptr, side = nullptr;
+    cudaEvent_t downloads = nullptr;  // side stream: everything enqueued before the last host bounce that stores directly
     uint64_t submitted = 0;
 };
 
@@ -95,6 +96,7 @@ extern "C" rr_status rr_pipeline_create(const rr_bvh *bvh, uint32_t max_n, const
     for (HostSlot &h : p->slot)
         for (cudaEvent_t *ev : {&h.rays_up, &h.pay_up, &h.consumed, &h.traced, &h.pay_down, &h.done})
             if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->downloads, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         rr_pipeline_destroy(p);
         return fail_cuda(e, "rr_pipeline_create: streams or events");
@@ -111,6 +113,7 @@ extern "C" rr_status rr_pipeline_destroy(rr_pipeline *p) {
     for (HostSlot &h : p->slot)
         for (cudaEvent_t ev : {h.rays_up, h.pay_up, h.consumed, h.traced, h.pay_down, h.done})
             if (ev) cudaEventDestroy(ev);
+    if (p->downloads) cudaEventDestroy(p->downloads);
     if (p->upload) cudaStreamDestroy(p->upload);
     if (p->side) cudaStreamDestroy(p->side);
     cudaFree(p->mem);
@@ -186,8 +189,9 @@ extern "C" rr_status rr_pipeline_run(rr_pipeline *p, const float *o_tmin, const 
 // computes.
 //
 // hits_direct: null, or the device address of hits_host, into which the trace
-// then stores the hits itself, after every earlier submission's downloads (one
-// of them may go to the same buffer).
+// then stores the hits itself, after every download enqueued so far (one of
+// them may go to the same buffer).  The side stream is asked, not the slots: a
+// submission that failed half-way has recorded no `done`.
 static rr_status submit_host(rr_pipeline *p, const float *o_host, const float *d_host, const uint32_t *payload_host,
                              uint32_t n, float *hits_host, float *hits_direct, uint32_t *payload_out_host,
                              void *stream, uint64_t *ticket) {
@@ -218,7 +222,9 @@ static rr_status submit_host(rr_pipeline *p, const float *o_host, const float *d
     sync.payload_ready = pay ? h.pay_up : nullptr;
     sync.payload_free = pay ? h.pay_down : nullptr;
     sync.consumed = h.consumed;
-    sync.hits_free = hits_direct ? p->slot[(k & 1) ^ 1].done : h.done;
+    if (hits_direct) e = cudaEventRecord(p->downloads, p->side);
+    if (e != cudaSuccess) return fail_cuda(e, "rr_pipeline_submit_host: record");
+    sync.hits_free = hits_direct ? p->downloads : h.done;
     rr_status st = run_bounce(p, h.o_in, h.d_in, pay ? h.payload_in : nullptr, n, hits_direct ? hits_direct : h.hits,
                               pay ? h.payload_sorted : nullptr, stream, sync);
     if (st != RR_OK) return st;

@@ -38,3 +38,30 @@ def test_direct_hits_match_staged(n, payload):
         assert not payload or np.array_equal(pay.numpy(), want_pay)
     assert rr.rr_device_error() == 0
     pipe.close()
+
+
+def test_direct_hits_wait_for_downloads_before_a_failed_submission():
+    """A submission still downloading, one that fails at its first launch, then a waiting bounce whose page-locked hits
+    lie at the end of the first one's: the last one's hits stay."""
+    big, n = 2_000_000, 33
+    tris = W.scene_box_soup(seed=2)
+    lo, hi = W.scene_aabb(tris)
+    bvh = rr.BVH(tris)
+    pipe = rr.Pipeline(bvh, big, rr.key_params(rr.RR_KEY_TWO_POINT, 32, lo, hi), radix_bits=8)
+    first, r = W.rays_box_soup(tris, n=big, seed=3), W.rays_box_soup(tris, n=n, seed=4)
+    o1, d1, o, d = [torch.from_numpy(a).pin_memory() for a in (first.o_tmin, first.d_tmax, r.o_tmin, r.d_tmax)]
+    want = np.zeros((n, 4), np.float32)
+    pipe.run_host(r.o_tmin, r.d_tmax, None, want, None)
+    hits, other = torch.full((big, 4), -7.0).pin_memory(), torch.zeros(n, 4).pin_memory()
+    for _ in range(3):
+        hits.fill_(-7.0)
+        pipe.submit_host(o1, d1, None, hits, None)
+        rr.rr_fault_inject("launch@1")
+        with pytest.raises(rr.RRError):
+            pipe.submit_host(o, d, None, other, None)
+        rr.rr_fault_inject(None)
+        pipe.run_host(o, d, None, hits[big - n:], None)
+        assert np.array_equal(hits[big - n:].numpy().view(np.uint32), want.view(np.uint32))
+        assert not (hits[:big - n] == -7.0).any()
+    assert rr.rr_device_error() == 0
+    pipe.close()
