@@ -27,6 +27,7 @@
 // out positions of an index buffer, so sorted rays are traced without being
 // gathered first, Section 4.4.1) and any-hit traversal for shadow rays (the first
 // triangle found inside the interval ends the ray, Section 4).
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -1308,29 +1309,42 @@ void *trace_entry() {
     return QUAD ? (void *)trace_quad_kernel<ACC, ANY, MULTI, BLOCK> : (void *)trace_kernel<ACC, ANY, MULTI, BLOCK>;
 }
 
+// Blocks of a trace kernel that an SM holds, and that shared-memory size: one
+// word, so that callers on several threads see both of the same query.
 template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
-int trace_blocks_per_sm(size_t smem) {
-    static int bps = 0;
-    static size_t bps_smem = 0;
-    if (bps == 0 || bps_smem != smem) {  // the batch kernels' shared memory varies with the segments
-        int v = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &v, trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>(), BLOCK, smem);
-        bps = (e != cudaSuccess || v < 1) ? 1 : v;
-        bps_smem = smem;
+cudaError_t trace_blocks_per_sm(size_t smem, uint32_t *blocks) {
+    static std::atomic<uint64_t> known{0};  // smem << 16 | blocks
+    const uint64_t k = known.load(std::memory_order_relaxed);
+    if ((k & 0xFFFFu) != 0 && k >> 16 == smem) {  // the batch kernels' shared memory varies with the segments
+        *blocks = (uint32_t)(k & 0xFFFFu);
+        return cudaSuccess;
     }
-    return bps;
+    void *entry = trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>();
+    // Static and dynamic shared memory together may pass the default 48 KB: the
+    // limit is raised before the query, which finds no room for a block beyond it
+    // (one block per SM instead of two: 2M rays in 200 segments of a batch with
+    // 512-thread blocks 1161 us instead of 740).
+    if (MULTI) {
+        const cudaError_t e = cudaFuncSetAttribute(entry, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)multi_smem(kMaxBatchSegments));
+        if (e != cudaSuccess) return e;
+    }
+    int v = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, entry, BLOCK, smem);
+    if (e != cudaSuccess) return e;
+    *blocks = v < 1 ? 1u : (uint32_t)v;
+    if (v >= 1) known.store((uint64_t)smem << 16 | (uint64_t)v, std::memory_order_relaxed);
+    return cudaSuccess;
 }
 
+// An error stays the thread's last CUDA error, which the caller's check reports.
 template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
 void trace_enqueue_form(const TraceArgs &a, int sm_count, cudaStream_t s) {
     const size_t smem = MULTI ? multi_smem(a.n_segs) : 0;
     const uint32_t per_block = QUAD ? BLOCK / 4 : BLOCK;  // rays a block holds at a time
-    uint32_t grid = (uint32_t)sm_count * (uint32_t)trace_blocks_per_sm<QUAD, ACC, ANY, MULTI, BLOCK>(smem);
-    grid = std::max(1u, std::min(grid, (a.n + per_block - 1u) / per_block));
-    if (MULTI)  // static and dynamic shared memory together may pass the default 48 KB
-        cudaFuncSetAttribute(trace_entry<QUAD, ACC, ANY, MULTI, BLOCK>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)multi_smem(kMaxBatchSegments));
+    uint32_t bps = 0;
+    if (trace_blocks_per_sm<QUAD, ACC, ANY, MULTI, BLOCK>(smem, &bps) != cudaSuccess) return;
+    const uint32_t grid = std::max(1u, std::min((uint32_t)sm_count * bps, (a.n + per_block - 1u) / per_block));
     launch_dependent(QUAD ? trace_quad_kernel<ACC, ANY, MULTI, BLOCK> : trace_kernel<ACC, ANY, MULTI, BLOCK>, grid, BLOCK,
                      smem, s, a);
 }
