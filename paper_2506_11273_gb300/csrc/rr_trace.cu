@@ -35,6 +35,7 @@
 #include "rr_batch.cuh"
 #include "rr_common.cuh"
 #include "rr_keymath.cuh"
+#include "rr_reciprocal.cuh"
 #include "rr_trace.h"
 
 namespace rr {
@@ -65,19 +66,6 @@ struct TraceArgs {
     const uint32_t *seg_offsets;
     uint32_t n_segs;
 };
-
-// Reciprocal of a direction component, kept finite: the hardware estimate (1
-// ulp) and one Newton step in fused arithmetic, which rounds 1/m correctly
-// unless m's mantissa is all ones (Markstein, IBM J. Res. Dev. 34(1), 1990).
-// The rounded intrinsic gives the same box tests; its range checks, at the few
-// lanes of a refill, cost 3% of a camera-ray trace.
-__device__ __forceinline__ float safe_inv(float x) {
-    const float m = fabsf(x) > 1e-18f ? x : copysignf(1e-18f, x);
-    float y;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(m));
-    const float z = fmaf(y, fmaf(-m, y, 1.0f), y);
-    return y == 0.0f ? y : z;  // an infinite m
-}
 
 // Eight 32-bit words by one 256-bit load (32-byte aligned, read-only data).
 struct Words8 {
