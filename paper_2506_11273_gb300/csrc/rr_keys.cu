@@ -1,6 +1,7 @@
 // Sorting keys (Section 3.1, Figure 2) and the adaptive ray-length table
 // (Section 3.1.6).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 
@@ -102,9 +103,10 @@ __device__ __forceinline__ KeyT ray_key(const QuantFrame &f, float4 o, float4 d,
 constexpr int kKeyTile = 512;
 constexpr uint32_t kCopySpinLimit = 1u << 22;  // polls of a copy's barrier before giving up
 
-// Digit-count entries of the fused form: passes x 2^radix_bits <= 2048 for
-// every key width with 4- or 8-bit digits.
-constexpr int kCountEntries = 2048;
+// Digit-count entries of the fused form: passes x 2^radix_bits is at most 256
+// a key byte with 4- or 8-bit digits.
+template <typename KeyT>
+constexpr uint32_t kCountEntries = 256 * sizeof(KeyT);
 
 // Adds a key's digit of every sort pass to the counters.  Bits above the key's
 // are zero, so the last pass's digit needs no narrower mask.  8-bit digits at
@@ -126,10 +128,10 @@ __device__ __forceinline__ void count_digits(KeyT key, uint32_t *counts, uint32_
 // After a block's last key: its counts (two copies) go to the sort's digit
 // counts, two neighbouring 32-bit counts per 64-bit atomic (no count passes
 // 2^30), and the sort's look-back words and tile counters are cleared.
-__device__ __forceinline__ void finish_counts(const uint32_t (&s_cnt)[2][kCountEntries], const SortCountTarget &c) {
+__device__ __forceinline__ void finish_counts(const uint32_t *even, const uint32_t *odd, const SortCountTarget &c) {
     const uint32_t entries = c.passes << c.radix_bits;
     for (uint32_t i = 2 * threadIdx.x; i < entries; i += 2 * blockDim.x) {
-        const uint32_t c0 = s_cnt[0][i] + s_cnt[1][i], c1 = s_cnt[0][i + 1] + s_cnt[1][i + 1];
+        const uint32_t c0 = even[i] + odd[i], c1 = even[i + 1] + odd[i + 1];
         if (c0 | c1) atomicAdd(reinterpret_cast<unsigned long long *>(c.hist + i), (unsigned long long)c1 << 32 | c0);
     }
     if (blockIdx.x == 0 && threadIdx.x < c.passes) c.counters[threadIdx.x] = 0u;
@@ -141,13 +143,15 @@ __device__ __forceinline__ void finish_counts(const uint32_t (&s_cnt)[2][kCountE
 // every sort pass of its keys (shared atomics into two copies, even and odd
 // warps), adds its counts to the sort's digit counts once at the end, and
 // clears the sort's look-back words and tile counters, so the separate
-// counting kernel of the sort is not needed.
+// counting kernel of the sort is not needed.  The counters are dynamic shared
+// memory: beside the two ray buffers the 16 KB of 64-bit keys'
+// 8-bit digits pass the 48 KB that static shared memory is documented to reach.
 template <int LAYOUT, int TSRC, typename KeyT, bool COUNT>
 __global__ void __launch_bounds__(kKeyTile, 3) key_kernel(KeyArgs a) {
     __shared__ __align__(128) float4 s_o[2][kKeyTile];
     __shared__ __align__(128) float4 s_d[2][kKeyTile];
     __shared__ __align__(8) uint64_t s_bar[2];
-    __shared__ uint32_t s_cnt[COUNT ? 2 : 1][COUNT ? kCountEntries : 1];
+    extern __shared__ uint32_t s_cnt[];  // COUNT: even warps' counters, then odd warps'
     const uint32_t tid = threadIdx.x;
     const uint32_t tiles = (a.n + kKeyTile - 1) / kKeyTile;
     if (tid == 0) {
@@ -156,7 +160,7 @@ __global__ void __launch_bounds__(kKeyTile, 3) key_kernel(KeyArgs a) {
         mbar_init_fence();
     }
     if (COUNT)
-        for (uint32_t i = tid; i < 2u * kCountEntries; i += kKeyTile) (&s_cnt[0][0])[i] = 0u;
+        for (uint32_t i = tid; i < 2u * kCountEntries<KeyT>; i += kKeyTile) s_cnt[i] = 0u;
     const uint32_t *lut = block_spread6_lut();
     const QuantFrame f = block_frame(a.lo, a.hi);  // synchronises: barriers, counters and table published
     auto issue = [&](uint32_t t, uint32_t buf) {
@@ -191,13 +195,13 @@ __global__ void __launch_bounds__(kKeyTile, 3) key_kernel(KeyArgs a) {
             const KeyT key =
                 ray_key<LAYOUT, TSRC, KeyT>(f, s_o[buf][tid], s_d[buf][tid], a.bits, a.ratio, tg, a.table, lut);
             static_cast<KeyT *>(a.keys)[i] = key;
-            if (COUNT) count_digits(key, s_cnt[(tid >> 5) & 1u], a.count.passes, a.count.radix_bits);
+            if (COUNT) count_digits(key, s_cnt + ((tid >> 5) & 1u) * kCountEntries<KeyT>, a.count.passes, a.count.radix_bits);
         }
         __syncthreads();  // every thread is done with `buf` before it is refilled
     }
     if constexpr (COUNT) {
         __syncthreads();
-        finish_counts(s_cnt, a.count);
+        finish_counts(s_cnt, s_cnt + kCountEntries<KeyT>, a.count);
     }
 }
 
@@ -213,10 +217,10 @@ __global__ void __launch_bounds__(kKeyTile, 3) key_batch_kernel(const BatchScene
                                                                uint32_t bits, float ratio, KeyT *__restrict__ keys,
                                                                SortCountTarget count) {
     __shared__ uint32_t s_off[kMaxBatchSegments + 1];
-    __shared__ uint32_t s_cnt[2][kCountEntries];
+    __shared__ uint32_t s_cnt[2][kCountEntries<KeyT>];
     const uint32_t *lut = block_spread6_lut();
     for (uint32_t k = threadIdx.x; k <= n_segs; k += kKeyTile) s_off[k] = seg_offsets[k];
-    for (uint32_t k = threadIdx.x; k < 2u * kCountEntries; k += kKeyTile) (&s_cnt[0][0])[k] = 0u;
+    for (uint32_t k = threadIdx.x; k < 2u * kCountEntries<KeyT>; k += kKeyTile) (&s_cnt[0][0])[k] = 0u;
     __syncthreads();
     const uint32_t tiles = (n + kKeyTile - 1) / kKeyTile;
     for (uint32_t t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(kKeyTile, 3) key_batch_kernel(const BatchScene
         count_digits(key, s_cnt[(threadIdx.x >> 5) & 1u], count.passes, count.radix_bits);
     }
     __syncthreads();
-    finish_counts(s_cnt, count);
+    finish_counts(s_cnt[0], s_cnt[1], count);
 }
 
 __global__ void batch_frame_kernel(BatchScene *segs, const float *boxes, uint32_t n) {
@@ -250,29 +254,45 @@ __global__ void batch_frame_kernel(BatchScene *segs, const float *boxes, uint32_
     segs[k].invE = __fdiv_rn(1.0f, f.E);
 }
 
+// Dynamic shared memory of a key kernel: the counters of its COUNT form.
+template <typename KeyT, bool COUNT>
+constexpr uint32_t key_smem() {
+    return COUNT ? 2u * (uint32_t)sizeof(uint32_t) * kCountEntries<KeyT> : 0u;
+}
+
 // Blocks of one key-kernel variant that fit on the device at once (its
-// occupancy is queried once per variant).
+// occupancy is queried once per variant, after its shared-memory limit is set).
 template <int LAYOUT, int TSRC, typename KeyT, bool COUNT>
-static uint32_t key_grid(uint32_t tiles, int sm_count) {
-    static int bps = 0;
-    if (bps == 0) {
-        int v = 0;
-        const cudaError_t e =
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, key_kernel<LAYOUT, TSRC, KeyT, COUNT>, kKeyTile, 0);
-        bps = (e == cudaSuccess && v > 0) ? v : 1;
+static cudaError_t key_grid(uint32_t tiles, int sm_count, uint32_t *grid) {
+    static std::atomic<int> bps{0};
+    int v = bps.load(std::memory_order_relaxed);
+    if (v == 0) {
+        const auto kernel = key_kernel<LAYOUT, TSRC, KeyT, COUNT>;
+        constexpr uint32_t smem = key_smem<KeyT, COUNT>();
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kernel, kKeyTile, smem);
+        if (e != cudaSuccess) return e;
+        v = std::max(v, 1);
+        bps.store(v, std::memory_order_relaxed);
     }
-    return std::max(1u, std::min(tiles, (uint32_t)(sm_count * bps)));
+    *grid = std::max(1u, std::min(tiles, (uint32_t)(sm_count * v)));
+    return cudaSuccess;
+}
+
+// An error stays the thread's last CUDA error, which the caller's check reports.
+template <int LAYOUT, int TSRC, typename KeyT, bool COUNT>
+static void launch_keys_k(const KeyArgs &a, int sm_count, cudaStream_t s) {
+    uint32_t grid = 0;
+    if (key_grid<LAYOUT, TSRC, KeyT, COUNT>((a.n + kKeyTile - 1) / kKeyTile, sm_count, &grid) != cudaSuccess) return;
+    key_kernel<LAYOUT, TSRC, KeyT, COUNT><<<grid, kKeyTile, key_smem<KeyT, COUNT>(), s>>>(a);
 }
 
 template <int LAYOUT, int TSRC, bool COUNT>
 static void launch_keys_t(const KeyArgs &a, bool wide, int sm_count, cudaStream_t s) {
-    const uint32_t tiles = (a.n + kKeyTile - 1) / kKeyTile;
     if (wide)
-        key_kernel<LAYOUT, TSRC, unsigned long long, COUNT>
-            <<<key_grid<LAYOUT, TSRC, unsigned long long, COUNT>(tiles, sm_count), kKeyTile, 0, s>>>(a);
+        launch_keys_k<LAYOUT, TSRC, unsigned long long, COUNT>(a, sm_count, s);
     else
-        key_kernel<LAYOUT, TSRC, uint32_t, COUNT>
-            <<<key_grid<LAYOUT, TSRC, uint32_t, COUNT>(tiles, sm_count), kKeyTile, 0, s>>>(a);
+        launch_keys_k<LAYOUT, TSRC, uint32_t, COUNT>(a, sm_count, s);
 }
 
 template <int LAYOUT, int TSRC>
