@@ -38,7 +38,25 @@ KEY_BITS = 64
 RADIX_BITS = 8
 # algorithmic bytes per ray (reads + writes of the data a phase must touch)
 BYTES_KEY = 32 + 8
-BYTES_SORT = 8 + (KEY_BITS // RADIX_BITS) * 2 * (8 + 4) - 4   # 196 for 64-bit keys, 8-bit digits
+
+
+def sort_bytes(bits: int, radix: int) -> int:
+    """Bytes a key that rr_sort without key output reads and writes: the counting pass's read of the keys, then per
+    digit pass the key and, after the first, the index in, the key and the index out.  The pass that uses up the low
+    half of a 64-bit key writes its high half only, the passes after it move 32-bit keys, the last writes no key."""
+    width = 8 if bits > 32 else 4
+    passes = -(-bits // radix)
+    total = width
+    for p in range(passes):
+        total += width + (4 if p > 0 else 0) + 4
+        if width == 8 and p == 32 // radix - 1 and passes > 32 // radix:
+            width = 4
+        if p < passes - 1:
+            total += width
+    return total
+
+
+BYTES_SORT = sort_bytes(KEY_BITS, RADIX_BITS)   # 156 for 64-bit keys, 8-bit digits
 BYTES_GATHER = 4 + 36 + 36
 BYTES_TRACE = 32 + 16
 BYTES_ACCUM = 32 + 16
@@ -742,16 +760,14 @@ def run_sweep(args):
                     evs[4].record(stream)
 
             ph = timed(step, 5)
-            kb = 8 if bits > 32 else 4
-            passes = -(-bits // radix)
-            sort_bytes = n * (kb + passes * 2 * (kb + 4) - 4)
+            moved = n * sort_bytes(bits, radix)
             hbm, _ = peaks()
             rows.append({"key_bits": bits, "radix_bits": radix,
                          "key_ms": round(float(ph[0]), 4), "sort_ms": round(float(ph[1]), 4),
                          "gather_ms": round(float(ph[2]), 4), "trace_accum_ms": round(float(ph[3]), 4),
                          "sorted_e2e_mrays": round(n / (float(ph.sum()) * 1e-3) / 1e6, 1),
-                         "sort_gbs": round(sort_bytes / (float(ph[1]) * 1e-3) / 1e9, 1),
-                         "sort_frac_hbm": round(sort_bytes / (float(ph[1]) * 1e-3) / 1e9 / hbm, 3)})
+                         "sort_gbs": round(moved / (float(ph[1]) * 1e-3) / 1e9, 1),
+                         "sort_frac_hbm": round(moved / (float(ph[1]) * 1e-3) / 1e9 / hbm, 3)})
             del ws
         del keys
     # the direction-first Costa key (32 bits with the gather and with indirect
