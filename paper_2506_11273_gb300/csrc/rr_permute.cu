@@ -7,15 +7,89 @@ namespace rr {
 
 constexpr int kPermuteBlock = 256;
 constexpr int kPermuteItems = 2;  // rays per thread: more loads in flight per thread
+constexpr uint32_t kPermuteRays = kPermuteBlock * kPermuteItems;
 
+// Wavefronts too large for L2 are moved one array after the other.  With all
+// three at once the random reads touch 36 bytes a ray of source: a sector's
+// second ray comes when its sector has left L2, and every 16-byte read costs a
+// DRAM access of its own.  One array at a time keeps most of its sectors (133
+// MB of origins at 8.3M rays against 129 MB of L2) until their other rays are
+// read, for two more streaming reads of the permutation; outputs are written
+// evict-first so that they do not push the sources out.  The payload goes first:
+// it leaves room for the permutation, which the next array then finds in L2.
+// A tile of the permutation is moved in ROUNDS rounds of PER rays a thread, and
+// one array of it takes a block as long as all arrays of kPermuteRays rays.
 template <bool PAYLOAD>
-__global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *o_in, const float4 *d_in,
-                                                               const uint32_t *p_in, const uint32_t *perm,
-                                                               uint32_t n, float4 *o_out, float4 *d_out,
-                                                               uint32_t *p_out, uint32_t *err) {
-    allow_dependent_launch();
+struct PhaseTile {
+    static constexpr int kPhases = PAYLOAD ? 3 : 2, PER = PAYLOAD ? 3 : 4, ROUNDS = PAYLOAD ? 2 : 1;
+    static constexpr uint32_t kRays = kPermuteBlock * PER * ROUNDS;
+    static_assert(kRays == kPhases * kPermuteRays, "a tile's phases share its rays when they are moved at once");
+};
+
+template <int PER, int ROUNDS, bool KEEP, typename T>
+__device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, uint32_t n, T *out, uint32_t first,
+                                             uint32_t *err) {
+#pragma unroll 1
+    for (int q = 0; q < ROUNDS; ++q) {
+        const uint32_t base = first + q * (kPermuteBlock * PER) + threadIdx.x;
+        uint32_t src[PER];
+        T v[PER];
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t i = base + j * kPermuteBlock;
+            src[j] = i < n ? (KEEP ? perm[i] : __ldcs(perm + i)) : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t i = base + j * kPermuteBlock;
+            if (i < n && index_ok(src[j], n, err)) v[j] = in[src[j]];
+        }
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t i = base + j * kPermuteBlock;
+            if (i < n && (!kChecked || src[j] < n)) __stcs(out + i, v[j]);
+        }
+    }
+}
+
+// Whether a tile's rays are in order already, or nearly: the sources of its first
+// 32 lie within 256 rays of one another and some share a 32-byte sector (none
+// does where every other ray is left for later).  Their sectors are used up at
+// once, and phases would only read the permutation three times.  The same answer
+// in every warp of every phase.
+__device__ __forceinline__ bool tile_in_order(const uint32_t *perm, uint32_t first, uint32_t n) {
+    const uint32_t s = perm[min(first + (threadIdx.x & 31u), n - 1u)];
+    if (__reduce_max_sync(0xFFFFFFFFu, s) - __reduce_min_sync(0xFFFFFFFFu, s) >= 256u) return false;
+    const uint32_t sector = __match_any_sync(0xFFFFFFFFu, s >> 1);
+    return __any_sync(0xFFFFFFFFu, (sector & (sector - 1u)) != 0u);
+}
+
+// A block moves kPermuteRays rays, every array of them; PHASED: one array of a
+// tile, unless the tile is in order, whose rays the blocks of the phases share.
+template <bool PAYLOAD, bool PHASED>
+__global__ void __launch_bounds__(kPermuteBlock) permute_kernel(
+    const float4 *o_in, const float4 *d_in, const uint32_t *p_in, const uint32_t *perm, uint32_t n, float4 *o_out,
+    float4 *d_out, uint32_t *p_out, uint32_t tiles, uint32_t *err) {
+    if (!PHASED) allow_dependent_launch();
     wait_for_prerequisite();
-    const uint32_t base = blockIdx.x * (kPermuteBlock * kPermuteItems) + threadIdx.x;
+    uint32_t first = blockIdx.x * kPermuteRays;
+    if (PHASED) {
+        using Tile = PhaseTile<PAYLOAD>;
+        const uint32_t phase = blockIdx.x / tiles;
+        first = (blockIdx.x - phase * tiles) * Tile::kRays;
+        if (!tile_in_order(perm, first, n)) {
+            const uint32_t array = PAYLOAD ? phase : phase + 1u;
+            if (array == 0)
+                gather_phase<Tile::PER, Tile::ROUNDS, true>(p_in, perm, n, p_out, first, err);
+            else if (array == 1)
+                gather_phase<Tile::PER, Tile::ROUNDS, false>(o_in, perm, n, o_out, first, err);
+            else
+                gather_phase<Tile::PER, Tile::ROUNDS, false>(d_in, perm, n, d_out, first, err);
+            return;
+        }
+        first += phase * kPermuteRays;
+    }
+    const uint32_t base = first + threadIdx.x;
     uint32_t src[kPermuteItems];
 #pragma unroll
     for (int j = 0; j < kPermuteItems; ++j) {
@@ -44,58 +118,29 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(const float4 *o_
     }
 }
 
-// Wavefronts too large for L2 are moved one array after the other.  With all
-// three at once the random reads touch 36 bytes a ray of source: a sector's
-// second ray comes when its sector has left L2, and every 16-byte read costs a
-// DRAM access of its own.  One array at a time keeps most of its sectors (133
-// MB of origins at 8.3M rays against 129 MB of L2) until their other rays are
-// read, for two more streaming reads of the permutation; outputs are written
-// evict-first so that they do not push the sources out.  Measured, random
-// order with payload: 8.3M rays 0.384 -> 0.254 ms (1.65 -> 2.48 TB/s of the 76
-// bytes a ray it cannot do without), 4.1M 0.142 -> 0.090, 3.0M 0.085 -> 0.064;
-// pixel-ordered rays, 8.3M: 0.156 -> 0.146.
-constexpr int kPhaseItems = 4;  // rays per thread and array
-
-template <typename T>
-__device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, uint32_t n, T *out,
-                                             uint32_t block, uint32_t *err) {
-    const uint32_t base = block * (kPermuteBlock * kPhaseItems) + threadIdx.x;
-    uint32_t src[kPhaseItems];
-    T v[kPhaseItems];
-#pragma unroll
-    for (int j = 0; j < kPhaseItems; ++j) {
-        const uint32_t i = base + j * kPermuteBlock;
-        src[j] = i < n ? __ldcs(perm + i) : 0u;
-    }
-#pragma unroll
-    for (int j = 0; j < kPhaseItems; ++j) {
-        const uint32_t i = base + j * kPermuteBlock;
-        if (i < n && index_ok(src[j], n, err)) v[j] = in[src[j]];
-    }
-#pragma unroll
-    for (int j = 0; j < kPhaseItems; ++j) {
-        const uint32_t i = base + j * kPermuteBlock;
-        if (i < n && (!kChecked || src[j] < n)) __stcs(out + i, v[j]);
-    }
-}
-
-__global__ void __launch_bounds__(kPermuteBlock) permute_phased_kernel(
-    const float4 *o_in, const float4 *d_in, const uint32_t *p_in, const uint32_t *perm, uint32_t n, float4 *o_out,
-    float4 *d_out, uint32_t *p_out, uint32_t phase_blocks, uint32_t *err) {
-    wait_for_prerequisite();
-    const uint32_t phase = blockIdx.x / phase_blocks, block = blockIdx.x - phase * phase_blocks;
-    if (phase == 0)
-        gather_phase(o_in, perm, n, o_out, block, err);
-    else if (phase == 1)
-        gather_phase(d_in, perm, n, d_out, block, err);
-    else
-        gather_phase(p_in, perm, n, p_out, block, err);
-}
-
 // From this many rays on (75 MB of sources, and as much of results) the phases
-// pay: at 2.07M rays 0.0455 against 0.0475 ms in random order, at 1.2M 0.0285
-// against 0.0265 in pixel order.
+// pay.  us with payload, buffers used in turn, all arrays at once / phases:
+// random order 2.1M rays 43.6 / 42.2, 2.6M 62.8 / 51.0, 4.1M 135 / 85, 8.3M 380 /
+// 250; pixel-ordered rays by a direction-first key 40.9 / 40.0, 56.2 / 48.5, 117 /
+// 79, 327 / 218, by a Two Point key 36.5 / 37.4, 44.9 / 45.6, 69.5 / 69.4, 152 / 142;
+// rays in order already 25.1 / 26.5, 30.3 / 32.1, 46.5 / 48.3, 91.2 / 93.8 (with no
+// test for them 27.5, 33.5, 51.9, 103.5); shuffled within 65,536 rays 35.3 / 37.6,
+// 42.6 / 45.9, 64.6 / 69.8, 125 / 135.
 constexpr uint32_t kPhasedRays = 1u << 21;
+
+template <bool PAYLOAD>
+static void launch_permute(const float4 *o_in, const float4 *d_in, const uint32_t *p_in, const uint32_t *perm, uint32_t n,
+                           float4 *o_out, float4 *d_out, uint32_t *p_out, uint32_t *err, cudaStream_t s) {
+    using Tile = PhaseTile<PAYLOAD>;
+    if (n >= kPhasedRays) {
+        const uint32_t tiles = (n + Tile::kRays - 1) / Tile::kRays;
+        launch_dependent(permute_kernel<PAYLOAD, true>, tiles * Tile::kPhases, kPermuteBlock, 0, s, o_in, d_in, p_in, perm,
+                         n, o_out, d_out, p_out, tiles, err);
+    } else {
+        launch_dependent(permute_kernel<PAYLOAD, false>, (n + kPermuteRays - 1) / kPermuteRays, kPermuteBlock, 0, s, o_in,
+                         d_in, p_in, perm, n, o_out, d_out, p_out, 0u, err);
+    }
+}
 
 }  // namespace rr
 
@@ -128,15 +173,10 @@ extern "C" rr_status rr_permute(const float *o_tmin_in, const float *d_tmax_in, 
     float4 *oo = reinterpret_cast<float4 *>(o_tmin_out);
     float4 *dd = reinterpret_cast<float4 *>(d_tmax_out);
     uint32_t *err = error_word(ds, s);
-    const uint32_t blocks = (n + kPermuteBlock * kPermuteItems - 1) / (kPermuteBlock * kPermuteItems);
-    if (n >= kPhasedRays) {
-        const uint32_t phase_blocks = (n + kPermuteBlock * kPhaseItems - 1) / (kPermuteBlock * kPhaseItems);
-        launch_dependent(permute_phased_kernel, phase_blocks * (payload_in ? 3u : 2u), kPermuteBlock, 0, s, oi, di,
-                         payload_in, perm, n, oo, dd, payload_out, phase_blocks, err);
-    } else {
-        launch_dependent(payload_in ? permute_kernel<true> : permute_kernel<false>, blocks, kPermuteBlock, 0, s, oi, di,
-                         payload_in, perm, n, oo, dd, payload_out, err);
-    }
+    if (payload_in)
+        launch_permute<true>(oi, di, payload_in, perm, n, oo, dd, payload_out, err, s);
+    else
+        launch_permute<false>(oi, di, nullptr, perm, n, oo, dd, nullptr, err, s);
     note_launches(1);
     return check_launch("rr_permute");
 }

@@ -34,7 +34,7 @@ KERNELS = list(_waiting_kernels())
 def test_every_waiting_kernel_is_found():
     calls = sum(_source(os.path.basename(p)).count("wait_for_prerequisite();")
                 for p in glob.glob(os.path.join(CSRC, "*.cu")))
-    assert len(KERNELS) == calls >= 6
+    assert len(KERNELS) == calls >= 5  # sort pass, reorder, table update, two traces
 
 
 @pytest.mark.parametrize("k", range(len(KERNELS)))
