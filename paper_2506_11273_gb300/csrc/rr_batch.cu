@@ -98,7 +98,7 @@ rr_status enqueue_batch(rr_batch *b, const float *o, const float *d, float *hits
                                      sm_count, s);
     if (st != RR_OK) return st;
     st = sort_enqueue_passes(b->keys, nullptr, perm, b->n_total, c.key_bits + b->seg_bits, c.radix_bits, b->sort_ws,
-                             err, s);
+                             err, sm_count, s);
     if (st != RR_OK) return st;
     return launch_trace_batch(b->d_segs, b->d_offsets, b->n_fronts, o, d, perm, b->n_total, hits, accumulating(b),
                               c.trace_block, b->queue, err, s);

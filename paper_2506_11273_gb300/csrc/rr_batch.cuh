@@ -59,11 +59,11 @@ struct SortCountTarget {
     uint32_t passes;
     uint32_t radix_bits;
 };
-SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits, void *workspace);
+SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits, void *workspace, int sm_count);
 
 // The digit passes of rr_sort once the counting stage has filled the
 // workspace (arguments already checked).
 rr_status sort_enqueue_passes(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
-                              uint32_t radix_bits, void *workspace, uint32_t *err, cudaStream_t s);
+                              uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s);
 
 }  // namespace rr

@@ -413,7 +413,7 @@ rr_status launch_keys_batch(const BatchScene *segs, const uint32_t *seg_offsets,
     const bool wide = key_bits + seg_bits > 32;
     const float4 *o = reinterpret_cast<const float4 *>(o_tmin);
     const float4 *d = reinterpret_cast<const float4 *>(d_tmax);
-    const SortCountTarget count = sort_count_target(n, key_bits + seg_bits, radix_bits, sort_workspace);
+    const SortCountTarget count = sort_count_target(n, key_bits + seg_bits, radix_bits, sort_workspace, sm_count);
     const cudaError_t e = cudaMemsetAsync(count.hist, 0, sizeof(uint32_t) * (count.passes << radix_bits), s);
     if (e != cudaSuccess) return fail_cuda(e, "rr_batch keys: memset");
 #define RR_KB(L, T)                                                                                              \
@@ -545,14 +545,14 @@ extern "C" rr_status rr_key_sort(const float *o_tmin, const float *d_tmax, uint3
     if (!ds) return st;
     cudaStream_t s = as_stream(stream);
     a.err = error_word(ds, s);
-    a.count = sort_count_target(n, p->bits, radix_bits, workspace);
+    a.count = sort_count_target(n, p->bits, radix_bits, workspace, ds->sm_count);
     const cudaError_t e = cudaMemsetAsync(a.count.hist, 0, sizeof(uint32_t) * (a.count.passes << radix_bits), s);
     if (e != cudaSuccess) return fail_cuda(e, "rr_key_sort: memset");
     launch_layout(p, a, true, ds->sm_count, s);
     note_launches(1);
     st = check_launch("rr_key_sort");
     if (st != RR_OK) return st;
-    return sort_enqueue_passes(keys_out, nullptr, perm_out, n, p->bits, radix_bits, workspace, a.err, s);
+    return sort_enqueue_passes(keys_out, nullptr, perm_out, n, p->bits, radix_bits, workspace, a.err, ds->sm_count, s);
 }
 
 extern "C" rr_status rr_length_table_create(const float lo[3], const float hi[3], rr_length_table **out,

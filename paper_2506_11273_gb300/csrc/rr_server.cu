@@ -212,7 +212,7 @@ rr_status launch_group(rr_server *s, Group *g) {
                                s->sm_count, st);
         if (rs == RR_OK)
             rs = sort_enqueue_passes(keys, nullptr, perm, (uint32_t)n, total_bits, s->cfg.radix_bits, wsp, sl.err,
-                                     st);
+                                     s->sm_count, st);
         if (rs == RR_OK)
             rs = launch_trace_batch(segs, offs, ng, o, d, perm, (uint32_t)n, hits, adaptive(s),
                                     s->cfg.trace_block, sl.queue, sl.err, st);

@@ -545,11 +545,9 @@ struct SortPlan {
     uint32_t tiles;   // its tiles
     uint32_t wb;      // bytes of a look-back word
     uint32_t regions; // sets of look-back words: a pass clears the set of the pass after it
+    uint32_t wave, wave4; // tiles that fit on the device at three and at four blocks per SM
     size_t off_hist, off_counters, off_lookback, off_keys_a, off_keys_b, off_vals, total;
 };
-
-// Tiles of a pass that fit on the device at three and four blocks per SM (152 SMs).
-constexpr uint32_t kWaveTiles = 456, kWaveTiles4 = 608;
 
 constexpr uint32_t full_items(uint32_t kb) {
     return kb == 8 ? SortTile<unsigned long long>::kItems : SortTile<uint32_t>::kItems;
@@ -564,8 +562,10 @@ constexpr uint32_t full_items(uint32_t kb) {
 // of it proportional to the keys of a thread (ranking, scatter), so the keys
 // are spread over as many tiles as still run at once: 4 keys per thread, then
 // 8, 12 and (32-bit keys) 16.  (64-bit words would not fit the smallest tiles
-// into the workspace, hence the 32-bit ones.)
-constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits) {
+// into the workspace, hence the 32-bit ones.)  Sizes and offsets in the workspace
+// do not depend on the device's SMs, only the tile size and with it the part of
+// the look-back words in use.
+constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits, int sm_count) {
     SortPlan p{};
     p.passes = (bits + radix_bits - 1) / radix_bits;
     p.radix = 1u << radix_bits;
@@ -576,10 +576,12 @@ constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits) {
     p.tiles = full_tiles;
     p.wb = 8;
     p.regions = p.passes > 1 ? 2u : 1u;
+    p.wave = 3u * (uint32_t)sm_count;
+    p.wave4 = 4u * (uint32_t)sm_count;
     for (uint32_t items = 4; items < full_items(p.kb); items += 4) {
         const uint32_t wb = items < 12 ? 4u : 8u;
         const uint32_t tiles = (n + kSortBlock * items - 1) / (kSortBlock * items);
-        if ((wb == 4 && n >= kSmallSortKeys) || tiles > kWaveTiles ||
+        if ((wb == 4 && n >= kSmallSortKeys) || tiles > p.wave ||
             (uint64_t)wb * p.regions * tiles > 8ull * p.passes * full_tiles)
             continue;
         p.items = items;
@@ -604,6 +606,12 @@ constexpr SortPlan plan_sort(uint32_t n, uint32_t bits, uint32_t radix_bits) {
     return p;
 }
 
+// Fewer SMs get larger tiles in place of a second wave, in the same workspace.
+static_assert(plan_sort(400000, 32, 8, 152).items == 4 && plan_sort(400000, 32, 8, 76).items == 8 &&
+                  plan_sort(400000, 32, 8, 76).tiles <= 3 * 76 && plan_sort(1100000, 64, 8, 76).tiles > 3 * 76 &&
+                  plan_sort(400000, 32, 8, 152).total == plan_sort(400000, 32, 8, 76).total,
+              "a plan is made for the SMs of its device");
+
 // 16-byte words of a plan's look-back words, which start at zero.
 constexpr size_t lookback_uint4(const SortPlan &p) { return (size_t)p.regions * p.tiles * p.radix * p.wb / 16; }
 
@@ -625,7 +633,7 @@ static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
 // The pass in the plan's tile size (for 64-bit plans also the passes over the
 // 32-bit high halves).  Full-size passes of more than one wave take the
 // four-block form, unless larger tiles keep the pass to one wave: 20 keys at
-// three blocks for 32-bit keys (1.87M to 2.33M keys; keys and sort of 1.9M 92.4
+// three blocks for 32-bit keys (1.87M to 2.33M keys on 152 SMs; keys and sort of 1.9M 92.4
 // -> 86.4 us, 2.07M 95.3 -> 90.9, 2.3M 97.9 -> 92.0, but 2.6M 115.6 -> 118.3), 14
 // keys at four blocks for 64-bit keys (1.87M to 2.18M; with the 32-bit passes
 // over their high halves 1.9M 182 -> 174 us, 2.07M 194 -> 176, but 1.7M 149 -> 162
@@ -637,16 +645,16 @@ static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaS
     if (pl.items == 4) return launch_pass<K, RBITS, 4, uint32_t, 3>(a, s);
     if (pl.items == 8) return launch_pass<K, RBITS, 8, uint32_t, 3>(a, s);
     const uint32_t tiles12 = (a.n + kSortBlock * 12 - 1) / (kSortBlock * 12);
-    if (tiles12 <= kWaveTiles && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
+    if (tiles12 <= pl.wave && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
     constexpr int FULL = SortTile<K>::kItems;
     const uint32_t tiles = (a.n + kSortBlock * FULL - 1) / (kSortBlock * FULL);
     if constexpr (RBITS == 8) {  // (4-bit digits: not measured)
         constexpr int LARGE = sizeof(K) == 8 ? 14 : 20;
-        constexpr uint32_t kWave = sizeof(K) == 8 ? kWaveTiles4 : kWaveTiles;
-        if (tiles > kWave && (a.n + kSortBlock * LARGE - 1) / (kSortBlock * LARGE) <= kWave)
+        const uint32_t wave = sizeof(K) == 8 ? pl.wave4 : pl.wave;
+        if (tiles > wave && (a.n + kSortBlock * LARGE - 1) / (kSortBlock * LARGE) <= wave)
             return launch_pass<K, RBITS, LARGE, W64, sizeof(K) == 8 ? 4 : 3>(a, s);
     }
-    if (tiles > kWaveTiles) return launch_pass<K, RBITS, FULL, W64, 4>(a, s);
+    if (tiles > pl.wave) return launch_pass<K, RBITS, FULL, W64, 4>(a, s);
     return launch_pass<K, RBITS, FULL, W64, 3>(a, s);
 }
 
@@ -764,7 +772,7 @@ static rr_status run_sort(const SortPlan &pl, const K *keys_in, K *keys_out, uin
 // The sort of rr_sort (arguments already checked).
 static rr_status sort_enqueue(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
                               uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s) {
-    const SortPlan pl = plan_sort(n, bits, radix_bits);
+    const SortPlan pl = plan_sort(n, bits, radix_bits, sm_count);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     if (pl.kb == 4) {
         const uint32_t *ki = static_cast<const uint32_t *>(keys_in);
@@ -778,8 +786,8 @@ static rr_status sort_enqueue(const void *keys_in, void *keys_out, uint32_t *per
                            : run_sort<unsigned long long, 4>(pl, ki, ko, perm_out, n, bits, ws, err, sm_count, s);
 }
 
-SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits, void *workspace) {
-    const SortPlan pl = plan_sort(n, bits, radix_bits);
+SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits, void *workspace, int sm_count) {
+    const SortPlan pl = plan_sort(n, bits, radix_bits, sm_count);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     SortCountTarget t;
     t.hist = reinterpret_cast<uint32_t *>(ws + pl.off_hist);
@@ -792,8 +800,8 @@ SortCountTarget sort_count_target(uint32_t n, uint32_t bits, uint32_t radix_bits
 }
 
 rr_status sort_enqueue_passes(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n, uint32_t bits,
-                              uint32_t radix_bits, void *workspace, uint32_t *err, cudaStream_t s) {
-    const SortPlan pl = plan_sort(n, bits, radix_bits);
+                              uint32_t radix_bits, void *workspace, uint32_t *err, int sm_count, cudaStream_t s) {
+    const SortPlan pl = plan_sort(n, bits, radix_bits, sm_count);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     cudaError_t e;
     if (pl.kb == 4) {
@@ -822,7 +830,7 @@ rr_status sort_check(const char *what, const void *keys_in, const void *keys_out
     if (n >= (1u << 30)) return fail(RR_ERR_INVALID_ARG, w + ": n must be < 2^30");
     if (n == 0) return RR_OK;
     if (!keys_in || !perm_out || !workspace) return fail(RR_ERR_INVALID_ARG, w + ": NULL buffer");
-    const SortPlan pl = plan_sort(n, bits, radix_bits);
+    const SortPlan pl = plan_sort(n, bits, radix_bits, 1);  // for its sizes
     if (workspace_bytes < pl.total) return fail(RR_ERR_INVALID_ARG, w + ": workspace too small");
     if (!aligned(workspace, 256)) return fail(RR_ERR_INVALID_ARG, w + ": workspace not 256-byte aligned");
     const size_t kbytes = (size_t)pl.kb * n;
@@ -846,7 +854,7 @@ extern "C" rr_status rr_sort_workspace_size(uint32_t n, uint32_t bits, uint32_t 
     if (radix_bits != 4 && radix_bits != 8)
         return fail(RR_ERR_INVALID_ARG, "rr_sort_workspace_size: radix_bits must be 4 or 8");
     if (n >= (1u << 30)) return fail(RR_ERR_INVALID_ARG, "rr_sort_workspace_size: n must be < 2^30");
-    *bytes = plan_sort(n, bits, radix_bits).total;
+    *bytes = plan_sort(n, bits, radix_bits, 1).total;
     return RR_OK;
 }
 
@@ -903,7 +911,7 @@ extern "C" rr_status rr_selftest_lookback_timeout(void *stream) {
     using K = uint32_t;
     constexpr uint32_t tile = kSortBlock * SortTile<K>::kItems;
     const uint32_t n = 2 * tile;
-    const SortPlan pl = plan_sort(n, 8, 8);  // (its full-size tile form is run here whatever the plan prefers)
+    const SortPlan pl = plan_sort(n, 8, 8, ds->sm_count);  // (its full-size tile form is run here whatever the plan prefers)
     unsigned char *ws = nullptr;
     K *keys = nullptr, *keys_out = nullptr;
     uint32_t *perm = nullptr;
@@ -957,10 +965,10 @@ constexpr size_t cx_max(size_t a, size_t b) { return a > b ? a : b; }
 
 constexpr size_t kNoAllocHeader = 256;  // device error word of this entry point
 constexpr size_t kNoAllocScratchBytes =
-    kNoAllocHeader + cx_max(cx_max(plan_sort(RR_SORT_NOALLOC_MAX_N, 64, 8).total,
-                                   plan_sort(RR_SORT_NOALLOC_MAX_N, 64, 4).total),
-                            cx_max(plan_sort(RR_SORT_NOALLOC_MAX_N, 32, 8).total,
-                                   plan_sort(RR_SORT_NOALLOC_MAX_N, 32, 4).total));
+    kNoAllocHeader + cx_max(cx_max(plan_sort(RR_SORT_NOALLOC_MAX_N, 64, 8, 1).total,
+                                   plan_sort(RR_SORT_NOALLOC_MAX_N, 64, 4, 1).total),
+                            cx_max(plan_sort(RR_SORT_NOALLOC_MAX_N, 32, 8, 1).total,
+                                   plan_sort(RR_SORT_NOALLOC_MAX_N, 32, 4, 1).total));
 static_assert(kNoAllocScratchBytes <= RR_SORT_NOALLOC_SCRATCH_BYTES, "scratch bound in rr.h is too small");
 
 static __device__ __align__(256) unsigned char g_sort_scratch[RR_SORT_NOALLOC_SCRATCH_BYTES];
@@ -1035,7 +1043,7 @@ extern "C" rr_status rr_sort_noalloc(const void *keys_in, void *keys_out, uint32
     if (n > RR_SORT_NOALLOC_MAX_N) return RR_ERR_TOO_LARGE;
     if (n == 0) return RR_OK;
     if (!keys_in || !perm_out) return RR_ERR_INVALID_ARG;
-    const SortPlan pl = plan_sort(n, bits, radix_bits);
+    SortPlan pl = plan_sort(n, bits, radix_bits, 1);  // for its sizes
     if (kNoAllocHeader + pl.total > sizeof(g_sort_scratch)) return RR_ERR_TOO_LARGE;
     const size_t kbytes = (size_t)pl.kb * n;
     if (!aligned(keys_in, pl.kb) || (keys_out && !aligned(keys_out, pl.kb)) || !aligned(perm_out, 4))
@@ -1046,6 +1054,7 @@ extern "C" rr_status rr_sort_noalloc(const void *keys_in, void *keys_out, uint32
     NoAllocDevice *d = nullptr;
     const rr_status st = noalloc_device(&d);
     if (st != RR_OK) return st;
+    pl = plan_sort(n, bits, radix_bits, d->sm_count);
     cudaStream_t s = as_stream(stream);
     if (pl.kb == 4) {
         const uint32_t *ki = static_cast<const uint32_t *>(keys_in);
