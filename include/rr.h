@@ -34,6 +34,16 @@
  *    device memory behind them.
  *  - Work is enqueued on `stream` (a cudaStream_t; NULL is the legacy default
  *    stream) and the call returns without synchronising, unless stated otherwise.
+ *  - Early launch: the sorts, rr_permute, the traces (with their table updates),
+ *    rr_pipeline_run and rr_batch_run overlap launch and drain of their kernels by
+ *    programmatic dependent launch, and the last kernel of such a call may let the
+ *    next kernel of `stream` start early.  A caller's own kernel launched there
+ *    with cudaLaunchAttributeProgrammaticStreamSerialization must call
+ *    cudaGridDependencySynchronize() before it reads or writes anything that an
+ *    earlier call on the stream reads or writes, and must then read results by
+ *    ordinary loads, not through the read-only path (__ldg, const __restrict__),
+ *    which needs data that stays unchanged for the kernel's whole life.  Kernels
+ *    launched without that attribute wait as usual.
  *  - Arguments are checked on the host before anything is enqueued.  A bad
  *    argument returns RR_ERR_INVALID_ARG and enqueues nothing.  n == 0 is a
  *    no-op that returns RR_OK.
@@ -176,12 +186,8 @@ rr_status rr_sort_workspace_size(uint32_t n, uint32_t bits, uint32_t radix_bits,
  * and perm_out must not overlap.  workspace: device, at least
  * rr_sort_workspace_size() bytes, 256-byte aligned, owned by the caller and
  * free again once the work on `stream` has completed.  n < 2^30.
- * One histogram pass plus ceil(bits / radix_bits) onesweep passes are enqueued;
- * the passes use programmatic dependent launch, and the last one lets the next
- * kernel of `stream` start early: a caller's kernel launched there with
- * cudaLaunchAttributeProgrammaticStreamSerialization must call
- * cudaGridDependencySynchronize() before it reads the sort's outputs (kernels
- * launched without that attribute wait for the sort as usual).
+ * One histogram pass plus ceil(bits / radix_bits) onesweep passes are enqueued
+ * (early launch: see the conventions above).
  */
 rr_status rr_sort(const void *keys_in, void *keys_out, uint32_t *perm_out, uint32_t n,
                   uint32_t bits, uint32_t radix_bits, void *workspace, size_t workspace_bytes,
