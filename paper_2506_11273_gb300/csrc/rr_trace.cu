@@ -577,6 +577,90 @@ __device__ __forceinline__ uint32_t quad_entry(uint32_t sp, uint32_t quad) {
     return (sp >> 2) * BLOCK + (sp & 3u) * 8u + quad;
 }
 
+// The next node group of a ray whose current one is used up; false: there is none.
+template <int BLOCK>
+__device__ __forceinline__ bool quad_pop(RayState &r, const uint2 *stack, uint32_t quad) {
+    if (r.sp == 0) return false;
+    --r.sp;
+    const uint2 e = stack[quad_entry<BLOCK>(r.sp, quad)];
+    r.g_base = e.x;
+    r.g_mask = e.y;
+    return true;
+}
+
+// Takes the nearest child of the current group and keeps the rest of the group
+// on the stack; false: the ray has to end.
+template <int BLOCK>
+__device__ __forceinline__ bool quad_take_child(RayState &r, uint2 *stack, uint32_t quad, const SceneRef &sc, uint32_t *err,
+                                                uint32_t &node) {
+    node = take_child(r);
+    bool ok = index_ok(node, sc.n_nodes, err);
+    if ((r.g_mask & 0xFFu) != 0u) {
+        if (r.sp < (int)kTraceStack) {
+            stack[quad_entry<BLOCK>(r.sp, quad)] = make_uint2(r.g_base, r.g_mask);  // the four lanes store the same
+        } else {
+            atomicOr(err, RR_DEVERR_TRACE_STACK);
+            ok = false;
+        }
+        ++r.sp;
+    }
+    return ok;
+}
+
+// The winner among the triangles that a ray's four lanes tested: the nearest
+// hit (ANY: the first), the first among equals.  True if one of them was hit.
+// All lanes of the warp call it; a lane without a hit has t infinite.
+template <bool ANY>
+__device__ __forceinline__ bool quad_winner(RayState &r, RegisterExtra &x, bool hit, float u, float v, float t, uint32_t k,
+                                            uint32_t quad, uint32_t j) {
+    const uint32_t hits = (__ballot_sync(0xFFFFFFFFu, hit) >> (4u * quad)) & 15u;
+    if (__any_sync(0xFFFFFFFFu, hit)) {
+        uint32_t win;
+        if (ANY) {
+            win = hits ? __ffs(hits) - 1u : 0u;
+        } else {
+            win = j;
+            float tw = t;
+#pragma unroll
+            for (int by = 1; by <= 2; by <<= 1) {
+                const float to = __shfl_xor_sync(0xFFFFFFFFu, tw, by);
+                const uint32_t wo = __shfl_xor_sync(0xFFFFFFFFu, win, by);
+                if (to < tw || (to == tw && wo < win)) {
+                    tw = to;
+                    win = wo;
+                }
+            }
+        }
+        const uint32_t from = 4u * quad + win;
+        const float tw = __shfl_sync(0xFFFFFFFFu, t, from), uw = __shfl_sync(0xFFFFFFFFu, u, from),
+                    vw = __shfl_sync(0xFFFFFFFFu, v, from);
+        const uint32_t kw = __shfl_sync(0xFFFFFFFFu, k, from);
+        if (hits != 0u) {
+            r.best = tw;
+            x.set_hit(uw, vw, kw);
+            if (ANY) ray_stop(r);
+        }
+    }
+    return hits != 0u;
+}
+
+// Whether the ray meets slot j + 4 * h of a node.
+__device__ __forceinline__ bool quad_slot(const RayState &r, const NodeSlabs &s, uint32_t j, int h) {
+    const uint32_t sel = 0x7540u | j;  // byte j, then the mantissa and exponent of 2^23
+    const auto at = [&](uint32_t w, float b, float a) {
+        return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), b, a);
+    };
+    const float t0 = max3f(at(s.nx[h], s.bx, s.ax), at(s.ny[h], s.by, s.ay), fmaxf(at(s.nz[h], s.bz, s.az), r.o.w));
+    const float t1 = min3f(at(s.fx[h], s.bx, s.ax), at(s.fy[h], s.by, s.ay), fminf(at(s.fz[h], s.bz, s.az), r.best));
+    return t0 <= t1;
+}
+
+// The hit slots of a ray's node from those of its lanes; all lanes of the warp call it.
+__device__ __forceinline__ uint32_t quad_slots(bool lo, bool hi, uint32_t quad) {
+    const uint32_t l = __ballot_sync(0xFFFFFFFFu, lo), h = __ballot_sync(0xFFFFFFFFu, hi);
+    return ((l >> (4u * quad)) & 15u) | (((h >> (4u * quad)) & 15u) << 4);
+}
+
 // One step: up to four pending triangles, or the next node.  Returns false
 // for the lanes of a ray that is finished (or of no ray).
 template <bool ANY, int BLOCK>
@@ -599,88 +683,30 @@ __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool li
             r.t.hits = h3 & (h3 - 1u);
             next_group(r, x);
         }
-        const uint32_t hits = (__ballot_sync(0xFFFFFFFFu, hit) >> (4u * quad)) & 15u;
-        if (__any_sync(0xFFFFFFFFu, hit)) {
-            // the winning lane of the four: the nearest hit (ANY: the first), the
-            // first among equals
-            uint32_t win;
-            if (ANY) {
-                win = hits ? __ffs(hits) - 1u : 0u;
-            } else {
-                win = j;
-                float tw = t;
-#pragma unroll
-                for (int by = 1; by <= 2; by <<= 1) {
-                    const float to = __shfl_xor_sync(0xFFFFFFFFu, tw, by);
-                    const uint32_t wo = __shfl_xor_sync(0xFFFFFFFFu, win, by);
-                    if (to < tw || (to == tw && wo < win)) {
-                        tw = to;
-                        win = wo;
-                    }
-                }
-            }
-            const uint32_t from = 4u * quad + win;
-            const float tw = __shfl_sync(0xFFFFFFFFu, t, from), uw = __shfl_sync(0xFFFFFFFFu, u, from),
-                        vw = __shfl_sync(0xFFFFFFFFu, v, from);
-            const uint32_t kw = __shfl_sync(0xFFFFFFFFu, k, from);
-            if (hits != 0u) {
-                r.best = tw;
-                x.set_hit(uw, vw, kw);
-                if (ANY) ray_stop(r);
-            }
-        }
+        quad_winner<ANY>(r, x, hit, u, v, t, k, quad, j);
     }
     __syncwarp();
     bool visit = live && r.t.hits == 0u, more = live;
-    if (visit && (r.g_mask & 0xFFu) == 0u) {
-        if (r.sp == 0) {
-            visit = false;
-            more = false;
-        } else {
-            --r.sp;
-            const uint2 e = stack[quad_entry<BLOCK>(r.sp, quad)];
-            r.g_base = e.x;
-            r.g_mask = e.y;
-        }
-    }
+    if (visit && (r.g_mask & 0xFFu) == 0u) visit = more = quad_pop<BLOCK>(r, stack, quad);
     Words8 n0{}, n2{};
     bool two[2] = {false, false};
     if (visit) {
-        const uint32_t node = take_child(r);
-        visit = index_ok(node, sc.n_nodes, err);
-        if ((r.g_mask & 0xFFu) != 0u) {
-            if (r.sp < (int)kTraceStack) {
-                stack[quad_entry<BLOCK>(r.sp, quad)] = make_uint2(r.g_base, r.g_mask);  // the four lanes store the same
-            } else {
-                atomicOr(err, RR_DEVERR_TRACE_STACK);
-                visit = false;
-            }
-            ++r.sp;
-        }
+        uint32_t node;
+        visit = quad_take_child<BLOCK>(r, stack, quad, sc, err, node);
         if (visit) {
             const DevNode *np = sc.nodes + node;
             n0 = load256(np);
             n2 = load256(&np->qlo_z);
             const NodeSlabs s = node_slabs(r, n0, load256(&np->qlo_x), n2);
-            const uint32_t sel = 0x7540u | j;  // byte j, then the mantissa and exponent of 2^23
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const auto at = [&](uint32_t w, float b, float a) {
-                    return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), b, a);
-                };
-                const float t0 = max3f(at(s.nx[h], s.bx, s.ax), at(s.ny[h], s.by, s.ay),
-                                       fmaxf(at(s.nz[h], s.bz, s.az), r.o.w));
-                const float t1 = min3f(at(s.fx[h], s.bx, s.ax), at(s.fy[h], s.by, s.ay),
-                                       fminf(at(s.fz[h], s.bz, s.az), r.best));
-                two[h] = t0 <= t1;
-            }
+            for (int h = 0; h < 2; ++h) two[h] = quad_slot(r, s, j, h);
         } else {
             x.set_hit(0.0f, 0.0f, kMiss);
             ray_stop(r);
         }
     }
-    const uint32_t lo = __ballot_sync(0xFFFFFFFFu, two[0]), hi = __ballot_sync(0xFFFFFFFFu, two[1]);
-    if (visit) take_hits(r, x, n0, n2, ((lo >> (4u * quad)) & 15u) | (((hi >> (4u * quad)) & 15u) << 4), tables);
+    const uint32_t hm = quad_slots(two[0], two[1], quad);
+    if (visit) take_hits(r, x, n0, n2, hm, tables);
     return more;
 }
 
@@ -691,44 +717,23 @@ __device__ __forceinline__ bool quad_step(RayState &r, RegisterExtra &x, bool li
 // compiled from one source disturb its main loop).  Returns as quad_step.
 template <bool ANY, int BLOCK>
 __device__ __forceinline__ bool quad_step_early(RayState &r, RegisterExtra &x, bool live, uint2 *stack, const SceneRef &sc,
-                                           uint32_t *err, const VisitTables &tables) {
-    constexpr int L = 4, P = 8 / L;
-    constexpr uint32_t LANES = (1u << L) - 1u;
-    const uint32_t lane = threadIdx.x & 31u, quad = lane / L, j = lane % L;
+                                                uint32_t *err, const VisitTables &tables) {
+    const uint32_t lane = threadIdx.x & 31u, quad = lane >> 2, j = lane & 3u;
     // the triangles this step tests, and the node it visits
     uint32_t left = r.t.hits, mine = left;
 #pragma unroll
-    for (uint32_t q = 0; q < (uint32_t)L; ++q) {
+    for (uint32_t q = 0; q < 4u; ++q) {
         if (q == j) mine = left;
         left &= left - 1u;
     }
     const bool test = live && r.t.hits != 0u;
     bool visit = live && (r.u_hits == 0u || left == 0u);
-    if (visit && (r.g_mask & 0xFFu) == 0u) {
-        if (r.sp == 0) {
-            visit = false;
-        } else {
-            --r.sp;
-            const uint2 e = stack[quad_entry<BLOCK>(r.sp, quad)];
-            r.g_base = e.x;
-            r.g_mask = e.y;
-        }
-    }
+    if (visit && (r.g_mask & 0xFFu) == 0u) visit = quad_pop<BLOCK>(r, stack, quad);
     const bool more = visit || test;
     Words8 n0{}, n1{}, n2{};
-    uint32_t node = 0u;
     if (visit) {
-        node = take_child(r);
-        visit = index_ok(node, sc.n_nodes, err);
-        if ((r.g_mask & 0xFFu) != 0u) {
-            if (r.sp < (int)kTraceStack) {
-                stack[quad_entry<BLOCK>(r.sp, quad)] = make_uint2(r.g_base, r.g_mask);  // its lanes store the same
-            } else {
-                atomicOr(err, RR_DEVERR_TRACE_STACK);
-                visit = false;
-            }
-            ++r.sp;
-        }
+        uint32_t node;
+        visit = quad_take_child<BLOCK>(r, stack, quad, sc, err, node);
         if (!visit) {
             x.set_hit(0.0f, 0.0f, kMiss);
             ray_stop(r);
@@ -752,60 +757,16 @@ __device__ __forceinline__ bool quad_step_early(RayState &r, RegisterExtra &x, b
             r.t.hits = left;
             next_group(r, x);
         }
-        const uint32_t hits = (__ballot_sync(0xFFFFFFFFu, hit) >> (L * quad)) & LANES;
-        if (__any_sync(0xFFFFFFFFu, hit)) {
-            // the winning lane: the nearest hit (ANY: the first), the first among equals
-            uint32_t win;
-            if (ANY) {
-                win = hits ? __ffs(hits) - 1u : 0u;
-            } else {
-                win = j;
-                float tw = t;
-#pragma unroll
-                for (int by = 1; by < L; by <<= 1) {
-                    const float to = __shfl_xor_sync(0xFFFFFFFFu, tw, by);
-                    const uint32_t wo = __shfl_xor_sync(0xFFFFFFFFu, win, by);
-                    if (to < tw || (to == tw && wo < win)) {
-                        tw = to;
-                        win = wo;
-                    }
-                }
-            }
-            const uint32_t from = L * quad + win;
-            const float tw = __shfl_sync(0xFFFFFFFFu, t, from), uw = __shfl_sync(0xFFFFFFFFu, u, from),
-                        vw = __shfl_sync(0xFFFFFFFFu, v, from);
-            const uint32_t kw = __shfl_sync(0xFFFFFFFFu, k, from);
-            if (hits != 0u) {
-                r.best = tw;
-                x.set_hit(uw, vw, kw);
-                if (ANY) {
-                    ray_stop(r);
-                    visit = false;
-                }
-            }
-        }
+        if (quad_winner<ANY>(r, x, hit, u, v, t, k, quad, j) && ANY) visit = false;
     }
     __syncwarp();
-    uint32_t in = 0u;  // bit i: slot j + L * i is hit
+    bool two[2] = {false, false};
     if (visit) {
         const NodeSlabs s = node_slabs(r, n0, n1, n2);
 #pragma unroll
-        for (int i = 0; i < P; ++i) {
-            // byte of slot j + L * i, then the mantissa and exponent of 2^23
-            const uint32_t sel = 0x7540u | (j + (uint32_t)((L * i) & 3));
-            const int h = (L * i) / 4;
-            const auto at = [&](uint32_t w, float b, float a) {
-                return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), b, a);
-            };
-            const float t0 = max3f(at(s.nx[h], s.bx, s.ax), at(s.ny[h], s.by, s.ay), fmaxf(at(s.nz[h], s.bz, s.az), r.o.w));
-            const float t1 = min3f(at(s.fx[h], s.bx, s.ax), at(s.fy[h], s.by, s.ay), fminf(at(s.fz[h], s.bz, s.az), r.best));
-            if (t0 <= t1) in |= 1u << i;
-        }
+        for (int h = 0; h < 2; ++h) two[h] = quad_slot(r, s, j, h);
     }
-    uint32_t hm = 0u;
-#pragma unroll
-    for (int i = 0; i < P; ++i)
-        hm |= ((__ballot_sync(0xFFFFFFFFu, (in >> i) & 1u) >> (L * quad)) & LANES) << (L * i);
+    const uint32_t hm = quad_slots(two[0], two[1], quad);
     if (visit) take_hits(r, x, n0, n2, hm, tables);
     return more;
 }
