@@ -630,32 +630,42 @@ static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
                             PassSmem<K, RBITS, ITEMS>::bytes, s, a);
 }
 
+// Rounds in which `tiles` tiles run on a device that holds `wave` of them; a few
+// beyond a full wave start as its first ones end and cost no round.
+constexpr uint32_t waves(uint32_t tiles, uint32_t wave, uint32_t spare) { return (tiles + wave - 1u - spare) / wave; }
+
 // The pass in the plan's tile size (for 64-bit plans also the passes over the
-// 32-bit high halves).  Full-size passes of more than one wave take the
-// four-block form, unless larger tiles keep the pass to one wave: 20 keys at
-// three blocks for 32-bit keys (1.87M to 2.33M keys on 152 SMs; keys and sort of 1.9M 92.4
-// -> 86.4 us, 2.07M 95.3 -> 90.9, 2.3M 97.9 -> 92.0, but 2.6M 115.6 -> 118.3), 14
-// keys at four blocks for 64-bit keys (1.87M to 2.18M; with the 32-bit passes
-// over their high halves 1.9M 182 -> 174 us, 2.07M 194 -> 176, but 1.7M 149 -> 162
-// and 2.3M 201 -> 207).  No pass has more tiles than the one before it, which
-// clears its look-back words.
+// 32-bit high halves).  Full-size passes that fit three blocks to an SM take that
+// form: its tiles are the fastest.  Beyond, larger tiles may keep the pass to one
+// wave: 20 keys at three blocks for 32-bit keys (1.88M to 2.33M keys on 152 SMs;
+// rr_sort of 1.9M 78.4 us against 84.4 and 85.7 at three and four blocks, of 2.07M
+// 80.9 against 93.6 and 85.6), 14 keys at four blocks for 64-bit keys (1.90M to
+// 2.18M; 2.16M 175 us against 189 and 184).  Else four blocks where they need
+// fewer waves than three, three where they need as many (us at three / four: 32-bit
+// keys 2.5M 103.5 / 95.8, 2.7M 106.6 / 112.6, 3.0M 114.1 / 120.3, 4.2M 144.7 / 141.1;
+// 64-bit 1.7M 174 / 150, 2.2M 196 / 209, 3.0M 247 / 240), and from two waves of four
+// on four (8.3M: 245 / 241, 600 / 577).
+// No pass has more tiles than the one before it, which clears its look-back words.
 template <typename K, int RBITS>
 static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaStream_t s) {
     using W64 = unsigned long long;
     if (pl.items == 4) return launch_pass<K, RBITS, 4, uint32_t, 3>(a, s);
     if (pl.items == 8) return launch_pass<K, RBITS, 8, uint32_t, 3>(a, s);
-    const uint32_t tiles12 = (a.n + kSortBlock * 12 - 1) / (kSortBlock * 12);
-    if (tiles12 <= pl.wave && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
-    constexpr int FULL = SortTile<K>::kItems;
-    const uint32_t tiles = (a.n + kSortBlock * FULL - 1) / (kSortBlock * FULL);
+    const auto tiles_of = [&](uint32_t items) { return (a.n + kSortBlock * items - 1) / (kSortBlock * items); };
+    const auto waves3 = [&](uint32_t items) { return waves(tiles_of(items), pl.wave, pl.wave / 100u); };
+    const auto waves4 = [&](uint32_t items) { return waves(tiles_of(items), pl.wave4, pl.wave4 / 50u); };
+    if (waves3(12) == 1 && (sizeof(K) == 8 || pl.items == 12)) return launch_pass<K, RBITS, 12, W64, 3>(a, s);
+    constexpr uint32_t FULL = SortTile<K>::kItems;
+    if (waves3(FULL) == 1) return launch_pass<K, RBITS, FULL, W64, 3>(a, s);
     if constexpr (RBITS == 8) {  // (4-bit digits: not measured)
-        constexpr int LARGE = sizeof(K) == 8 ? 14 : 20;
-        const uint32_t wave = sizeof(K) == 8 ? pl.wave4 : pl.wave;
-        if (tiles > wave && (a.n + kSortBlock * LARGE - 1) / (kSortBlock * LARGE) <= wave)
-            return launch_pass<K, RBITS, LARGE, W64, sizeof(K) == 8 ? 4 : 3>(a, s);
+        if constexpr (sizeof(K) == 4) {
+            if (tiles_of(20) <= pl.wave) return launch_pass<K, RBITS, 20, W64, 3>(a, s);
+        } else {
+            if (waves4(FULL) > 1 && tiles_of(14) <= pl.wave4) return launch_pass<K, RBITS, 14, W64, 4>(a, s);
+        }
     }
-    if (tiles > pl.wave) return launch_pass<K, RBITS, FULL, W64, 4>(a, s);
-    return launch_pass<K, RBITS, FULL, W64, 3>(a, s);
+    const bool four = waves4(FULL) < waves3(FULL) || tiles_of(FULL) >= 2u * pl.wave4;
+    return four ? launch_pass<K, RBITS, FULL, W64, 4>(a, s) : launch_pass<K, RBITS, FULL, W64, 3>(a, s);
 }
 
 // The counting stage of a sort: the digit counts of every pass start at zero
