@@ -206,7 +206,7 @@ struct PassArgs {
     const K *keys_in;
     const uint32_t *vals_in;  // null on the first pass: the value is the input index
     K *keys_out;              // null: keys are not written
-    uint32_t *high_out;       // 64-bit keys, not null: the keys' high halves are written here instead
+    uint32_t *high_out;       // 64-bit keys, keys_out null: the keys' high halves are written here (null: nothing)
     uint32_t *vals_out;
     uint32_t n;
     uint32_t shift;
@@ -235,8 +235,9 @@ static_assert(PassSmem<unsigned long long, 8, 12>::bytes <= 48 * 1024 && PassSme
 // One tile of a digit pass.  FULL tiles skip every bounds check; only the
 // last tile of a pass can be partial.  LATE loads the values after the
 // ranking (their loads then overlap the look-back), which keeps the ranking's
-// registers low enough for four blocks per SM.
-template <typename K, int RBITS, int ITEMS, typename W, bool FULL, bool LATE>
+// registers low enough for four blocks per SM.  ONCE asks what is written of
+// the keys (all, their high halves, nothing) once and not for every key.
+template <typename K, int RBITS, int ITEMS, typename W, bool ONCE, bool FULL, bool LATE>
 __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t tile, unsigned char *smem) {
     using Word = LookbackWord<W>;
     constexpr int RADIX = 1 << RBITS;
@@ -268,9 +269,15 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
             if (!LATE) v[j] = 0;
         }
     }
-    // while the keys arrive: the pass's digit counts, and the next pass's words cleared
+    // while the keys arrive: the pass's digit counts, and the next pass's words
+    // cleared; tiles of many keys clear them later, when fewer loads wait (32-bit
+    // keys beyond 1.5M 2% faster, sorts of 100,000 keys 3% slower)
+    constexpr bool CLEAR_EARLY = ITEMS <= 8 || RBITS == 4;
+    const auto clear_next = [&] {
+        if (a.lookback_next && tid < RADIX) static_cast<W *>(a.lookback_next)[(size_t)tile * RADIX + tid] = 0;
+    };
     const uint32_t total = tid < RADIX ? a.hist[tid] : 0u;
-    if (a.lookback_next && tid < RADIX) static_cast<W *>(a.lookback_next)[(size_t)tile * RADIX + tid] = 0;
+    if (CLEAR_EARLY) clear_next();
     // The tile's digit counts, published before the ranking so that later
     // tiles looking back wait on this tile's loads only, not on its ranking
     // (counts taken from the ranking instead: 1.2M 64-bit keys 0.137 -> 0.151 ms).
@@ -280,6 +287,7 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
     __syncthreads();
     const uint32_t cnt = tid < RADIX ? s_cnt[tid] : 0u;
     if (tid < RADIX) Word::store(row(tile), Word::make(tile, cnt));
+    if (!CLEAR_EARLY) clear_next();
 
     // stable rank inside the warp: items in index order (j, then lane).  The
     // peer masks of every row are independent; only the per-digit counters chain.
@@ -368,29 +376,44 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
     }
     __syncthreads();
     // global writes in tile order: runs of equal digits land contiguously
-    const auto put = [&](uint32_t i) {
-        const K key = s_keys[i];
-        const uint32_t gpos = s_gbase[digit_of(key, a.shift, a.mask)] + i;
-        if (!index_ok(gpos, a.n, a.err)) return;
-        if (sizeof(K) == 8 && a.high_out)
-            a.high_out[gpos] = (uint32_t)((unsigned long long)key >> 32);
-        else if (a.keys_out)
-            a.keys_out[gpos] = key;
-        a.vals_out[gpos] = s_vals[i];
-    };
-    if (FULL) {
+    const auto write = [&](auto &&put_key) {
+        const auto put = [&](uint32_t i) {
+            const K key = s_keys[i];
+            const uint32_t gpos = s_gbase[digit_of(key, a.shift, a.mask)] + i;
+            if (!index_ok(gpos, a.n, a.err)) return;
+            put_key(gpos, key);
+            a.vals_out[gpos] = s_vals[i];
+        };
+        if (FULL) {
 #pragma unroll
-        for (int j = 0; j < ITEMS; ++j) put(j * kSortBlock + tid);
+            for (int j = 0; j < ITEMS; ++j) put(j * kSortBlock + tid);
+        } else {
+            const uint32_t tile_n = min((uint32_t)TILE, a.n - base);
+            for (uint32_t i = tid; i < tile_n; i += kSortBlock) put(i);
+        }
+    };
+    const auto put_whole = [&](uint32_t at, K key) { a.keys_out[at] = key; };
+    const auto put_high = [&](uint32_t at, K key) { a.high_out[at] = (uint32_t)((unsigned long long)key >> 32); };
+    if (!ONCE) {
+        write([&](uint32_t at, K key) {
+            if (a.keys_out)
+                put_whole(at, key);
+            else if (sizeof(K) == 8 && a.high_out)
+                put_high(at, key);
+        });
+    } else if (a.keys_out) {
+        write(put_whole);
+    } else if (a.high_out) {
+        write(put_high);
     } else {
-        const uint32_t tile_n = min((uint32_t)TILE, a.n - base);
-        for (uint32_t i = tid; i < tile_n; i += kSortBlock) put(i);
+        write([](uint32_t, K) {});
     }
 }
 
 // MINB blocks per SM: 3 for passes of one wave or less (shortest tile
 // latency), 4 for longer passes (more tiles in flight).  Passes of four blocks
 // and of tiles above the full size load the values late.
-template <typename K, int RBITS, int ITEMS, typename W, int MINB>
+template <typename K, int RBITS, int ITEMS, typename W, int MINB, bool ONCE>
 __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> a) {
     using L = PassSmem<K, RBITS, ITEMS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -405,9 +428,9 @@ __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> 
     __syncthreads();
     const uint32_t tile = s_misc[0];
     if ((tile + 1) * (uint32_t)L::TILE <= a.n)
-        onesweep_tile<K, RBITS, ITEMS, W, true, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, ONCE, true, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
     else
-        onesweep_tile<K, RBITS, ITEMS, W, false, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
+        onesweep_tile<K, RBITS, ITEMS, W, ONCE, false, (MINB > 3 || ITEMS > SortTile<K>::kItems)>(a, tile, smem_raw);
 }
 
 // ------------------------------------------------------------------ local (segment) sort
@@ -617,15 +640,15 @@ constexpr size_t lookback_uint4(const SortPlan &p) { return (size_t)p.regions * 
 
 // One digit pass, launched so that it may start while the kernel before it
 // drains (programmatic dependent launch; the pass waits in the kernel).
-template <typename K, int RBITS, int ITEMS, typename W, int MINB>
+template <typename K, int RBITS, int ITEMS, typename W, int MINB, bool ONCE = false>
 static cudaError_t launch_pass(const PassArgs<K> &a, cudaStream_t s) {
     if (PassSmem<K, RBITS, ITEMS>::bytes > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(onesweep_kernel<K, RBITS, ITEMS, W, MINB>,
+        const cudaError_t e = cudaFuncSetAttribute(onesweep_kernel<K, RBITS, ITEMS, W, MINB, ONCE>,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)PassSmem<K, RBITS, ITEMS>::bytes);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(onesweep_kernel<K, RBITS, ITEMS, W, MINB>,
+    return launch_dependent(onesweep_kernel<K, RBITS, ITEMS, W, MINB, ONCE>,
                             (a.n + kSortBlock * ITEMS - 1) / (kSortBlock * ITEMS), kSortBlock,
                             PassSmem<K, RBITS, ITEMS>::bytes, s, a);
 }
@@ -644,7 +667,8 @@ constexpr uint32_t waves(uint32_t tiles, uint32_t wave, uint32_t spare) { return
 // fewer waves than three, three where they need as many (us at three / four: 32-bit
 // keys 2.5M 103.5 / 95.8, 2.7M 106.6 / 112.6, 3.0M 114.1 / 120.3, 4.2M 144.7 / 141.1;
 // 64-bit 1.7M 174 / 150, 2.2M 196 / 209, 3.0M 247 / 240), and from two waves of four
-// on four (8.3M: 245 / 241, 600 / 577).
+// on four (8.3M: 245 / 241, 600 / 577).  64-bit keys at three blocks beyond one wave
+// ask once what to write (2.2M 206 -> 196 us; the other forms lose 1 to 3% by it).
 // No pass has more tiles than the one before it, which clears its look-back words.
 template <typename K, int RBITS>
 static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaStream_t s) {
@@ -665,7 +689,7 @@ static cudaError_t dispatch_pass(const SortPlan &pl, const PassArgs<K> &a, cudaS
         }
     }
     const bool four = waves4(FULL) < waves3(FULL) || tiles_of(FULL) >= 2u * pl.wave4;
-    return four ? launch_pass<K, RBITS, FULL, W64, 4>(a, s) : launch_pass<K, RBITS, FULL, W64, 3>(a, s);
+    return four ? launch_pass<K, RBITS, FULL, W64, 4>(a, s) : launch_pass<K, RBITS, FULL, W64, 3, sizeof(K) == 8>(a, s);
 }
 
 // The counting stage of a sort: the digit counts of every pass start at zero
@@ -744,7 +768,7 @@ static cudaError_t enqueue_passes(const SortPlan &pl, const K *keys_in, K *keys_
             PassArgs<K> a{};
             fill(a);
             a.keys_in = kin;
-            a.keys_out = kout;
+            a.keys_out = p == drop ? nullptr : kout;
             a.high_out = p == drop ? reinterpret_cast<uint32_t *>(kout) : nullptr;
             a.shift = p * RBITS;
             e = dispatch_pass<K, RBITS>(pl, a, s);
@@ -948,7 +972,7 @@ extern "C" rr_status rr_selftest_lookback_timeout(void *stream) {
         a.lookback = ws + pl.off_lookback;
         a.tile_counter = counter;
         a.err = error_word(ds, s);
-        onesweep_kernel<K, 8, SortTile<K>::kItems, unsigned long long, 3>
+        onesweep_kernel<K, 8, SortTile<K>::kItems, unsigned long long, 3, false>
             <<<1, kSortBlock, PassSmem<K, 8, SortTile<K>::kItems>::bytes, s>>>(a);
         note_launches(1);
         e = cudaGetLastError();

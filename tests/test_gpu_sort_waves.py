@@ -22,7 +22,7 @@ def _keys(n, bits, seed):
 def test_sizes_around_the_waves(bits, radix, keys_out):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     tile = TILE[64 if bits > 32 else 32]
-    for tiles in (3 * sms, 3 * sms + 5, 4 * sms, 4 * sms + 13, 6 * sms + 5, 8 * sms):
+    for tiles in (3 * sms, 3 * sms + 5, 4 * sms, 4 * sms + 13, 5 * sms, 6 * sms + 5, 8 * sms):
         for n in (tiles * tile, tiles * tile + 1):
             k = _keys(n, bits, n)
             want, order = torch.sort(k, stable=True)
