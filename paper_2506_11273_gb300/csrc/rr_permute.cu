@@ -26,8 +26,20 @@ struct PhaseTile {
     static_assert(kRays == kPhases * kPermuteRays, "a tile's phases share its rays when they are moved at once");
 };
 
-template <int PER, int ROUNDS, bool KEEP, typename T>
-__device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, uint32_t n, T *out, uint32_t first,
+// Whether a warp's 32 rays are in order already, or nearly: their sources lie
+// within 40 rays of one another, so their sectors are used up at once and phases
+// would only read the permutation three times.  Sparser runs of sources, as coarse
+// keys of ordered rays leave them, are better moved in phases: 16-bit Aila keys of
+// 8.3M pixel-ordered rays 111 us with the line at 40, 116 at 64, 127 at 128.
+__device__ __forceinline__ bool row_in_order(uint32_t src) {
+    return __reduce_max_sync(0xFFFFFFFFu, src) - __reduce_min_sync(0xFFFFFFFFu, src) < 40u;
+}
+
+// One array of a tile.  ORDER: true, and nothing is moved, where the warp's first
+// row of the tile is in order; every array's block reads that row and finds the
+// same.
+template <int PER, int ROUNDS, bool KEEP, bool ORDER, typename T>
+__device__ __forceinline__ bool gather_phase(const T *in, const uint32_t *perm, uint32_t n, T *out, uint32_t first,
                                              uint32_t *err) {
 #pragma unroll 1
     for (int q = 0; q < ROUNDS; ++q) {
@@ -39,6 +51,7 @@ __device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, 
             const uint32_t i = base + j * kPermuteBlock;
             src[j] = i < n ? (KEEP ? perm[i] : __ldcs(perm + i)) : 0u;
         }
+        if (ORDER && q == 0 && (base | 31u) < n && row_in_order(src[0])) return true;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
             const uint32_t i = base + j * kPermuteBlock;
@@ -50,22 +63,13 @@ __device__ __forceinline__ void gather_phase(const T *in, const uint32_t *perm, 
             if (i < n && (!kChecked || src[j] < n)) __stcs(out + i, v[j]);
         }
     }
-}
-
-// Whether a tile's rays are in order already, or nearly: the sources of its first
-// 32 lie within 256 rays of one another and some share a 32-byte sector (none
-// does where every other ray is left for later).  Their sectors are used up at
-// once, and phases would only read the permutation three times.  The same answer
-// in every warp of every phase.
-__device__ __forceinline__ bool tile_in_order(const uint32_t *perm, uint32_t first, uint32_t n) {
-    const uint32_t s = perm[min(first + (threadIdx.x & 31u), n - 1u)];
-    if (__reduce_max_sync(0xFFFFFFFFu, s) - __reduce_min_sync(0xFFFFFFFFu, s) >= 256u) return false;
-    const uint32_t sector = __match_any_sync(0xFFFFFFFFu, s >> 1);
-    return __any_sync(0xFFFFFFFFu, (sector & (sector - 1u)) != 0u);
+    return false;
 }
 
 // A block moves kPermuteRays rays, every array of them; PHASED: one array of a
-// tile, unless the tile is in order, whose rays the blocks of the phases share.
+// tile, but for warps whose rays are in order: they move every array of their
+// share of the tile (with a payload; without one, two readings of the permutation
+// are not worth the question).
 // early: the next kernel of the stream may start now.
 template <bool PAYLOAD, bool PHASED>
 __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(
@@ -78,16 +82,15 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(
         using Tile = PhaseTile<PAYLOAD>;
         const uint32_t phase = blockIdx.x / tiles;
         first = (blockIdx.x - phase * tiles) * Tile::kRays;
-        if (!tile_in_order(perm, first, n)) {
-            const uint32_t array = PAYLOAD ? phase : phase + 1u;
-            if (array == 0)
-                gather_phase<Tile::PER, Tile::ROUNDS, true>(p_in, perm, n, p_out, first, err);
-            else if (array == 1)
-                gather_phase<Tile::PER, Tile::ROUNDS, false>(o_in, perm, n, o_out, first, err);
-            else
-                gather_phase<Tile::PER, Tile::ROUNDS, false>(d_in, perm, n, d_out, first, err);
-            return;
-        }
+        const uint32_t array = PAYLOAD ? phase : phase + 1u;
+        bool in_order;
+        if (array == 0)
+            in_order = gather_phase<Tile::PER, Tile::ROUNDS, true, PAYLOAD>(p_in, perm, n, p_out, first, err);
+        else if (array == 1)
+            in_order = gather_phase<Tile::PER, Tile::ROUNDS, false, PAYLOAD>(o_in, perm, n, o_out, first, err);
+        else
+            in_order = gather_phase<Tile::PER, Tile::ROUNDS, false, PAYLOAD>(d_in, perm, n, d_out, first, err);
+        if (!in_order) return;
         first += phase * kPermuteRays;
     }
     const uint32_t base = first + threadIdx.x;
@@ -121,12 +124,12 @@ __global__ void __launch_bounds__(kPermuteBlock) permute_kernel(
 
 // From this many rays on (75 MB of sources, and as much of results) the phases
 // pay.  us with payload, buffers used in turn, all arrays at once / phases:
-// random order 2.1M rays 43.6 / 42.2, 2.6M 62.8 / 51.0, 4.1M 135 / 85, 8.3M 380 /
-// 250; pixel-ordered rays by a direction-first key 40.9 / 40.0, 56.2 / 48.5, 117 /
-// 79, 327 / 218, by a Two Point key 36.5 / 37.4, 44.9 / 45.6, 69.5 / 69.4, 152 / 142;
-// rays in order already 25.1 / 26.5, 30.3 / 32.1, 46.5 / 48.3, 91.2 / 93.8 (with no
-// test for them 27.5, 33.5, 51.9, 103.5); shuffled within 65,536 rays 35.3 / 37.6,
-// 42.6 / 45.9, 64.6 / 69.8, 125 / 135.
+// random order 2.1M rays 43.4 / 42.2, 3.0M 78.5 / 58.9, 4.1M 129 / 85, 8.3M 354 /
+// 241; pixel-ordered rays by a direction-first key 40.6 / 40.1, 70.2 / 55.1, 113 /
+// 78, 309 / 212, by a Two Point key 36.5 / 37.4, 51.0 / 51.2, 69.0 / 68.6, 151 / 141;
+// rays in order already 24.9 / 26.6, 34.9 / 37.1, 46.7 / 49.9, 91.6 / 97.8 (with no
+// question for them 27.6, 38.1, 51.9, 103.7); shuffled within 65,536 rays 35.2 /
+// 37.6, 48.8 / 51.7, 64.8 / 69.1, 125 / 135.
 constexpr uint32_t kPhasedRays = 1u << 21;
 
 // Blocks that an SM holds, and blocks that leave nearly every SM free.  Only
