@@ -62,12 +62,13 @@ BYTES_TRACE = 32 + 16
 BYTES_ACCUM = 32 + 16
 TRACE_SOURCES = ["paper_2506_11273_gb300/csrc/rr_trace.cu", "paper_2506_11273_gb300/csrc/rr_trace.h",
                  "paper_2506_11273_gb300/csrc/rr_common.cuh", "paper_2506_11273_gb300/csrc/rr_bvh.cpp",
-                 "paper_2506_11273_gb300/csrc/rr_keymath.cuh", "paper_2506_11273_gb300/csrc/rr_batch.cuh"]
+                 "paper_2506_11273_gb300/csrc/rr_keymath.cuh", "paper_2506_11273_gb300/csrc/rr_batch.cuh",
+                 "paper_2506_11273_gb300/csrc/rr_reciprocal.cuh"]
 # One ncu capture of the trace kernel on this workload (bounce-3 wavefront, sorted
 # rays, `trace_kernel<0, 0, 0, 128>`): DRAM bytes read + written and warp
 # instructions per launch, valid only while the trace sources hash to `sources`
 # (sha256 of TRACE_SOURCES, first 16 hex digits); otherwise traffic is reported as null.
-TRACE_NCU = {"sources": "5adfdf8d3c13586f", "dram_bytes": 132669696 + 12462080, "warp_instructions": 376998630}
+TRACE_NCU = {"sources": "80879d034465a036", "dram_bytes": 132654848 + 11936768, "warp_instructions": 375855063}
 # issue-slot peak: 4 warp instructions per cycle per SM (one per scheduler) x 152 SMs
 SMS, ISSUE_PER_SM_CYCLE, MAX_SM_MHZ = 152, 4, 2070.0
 

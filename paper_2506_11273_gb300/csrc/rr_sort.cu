@@ -12,9 +12,10 @@
 // 1.0, look-back 1.7, shared scatter 1.8, writes 1.3, kernel boundary 1.2),
 // beyond that issue and latency together.  Hence tiles as small as one wave
 // allows (plan_sort), both scans behind one barrier, and 32-bit passes once a
-// 64-bit key's low half is used up.  Keys and sort together, before and after:
-// 4,097 32-bit keys 33 -> 23 us, 65,536 64-bit 71 -> 51, 689,149 32-bit 62 -> 56,
-// 1.2M 64-bit 134 -> 127, 2.07M 32-bit 108 -> 99, 8.3M 64-bit 617 -> 562.
+// 64-bit key's low half is used up.  Keys and sort together (rr_key_sort, Two Point
+// keys), with the passes before these and now: 4,097 32-bit keys 29.6 -> 24.7 us,
+// 65,536 64-bit 67 -> 48, 300,001 64-bit 83.5 -> 69.6, 689,149 32-bit 61 -> 50, 1.2M
+// 64-bit 131 -> 121, 2.07M 32-bit 106 -> 88, 8.3M 64-bit 629 -> 558.
 #include <algorithm>
 #include <mutex>
 
@@ -410,9 +411,9 @@ __device__ __forceinline__ void onesweep_tile(const PassArgs<K> &a, uint32_t til
     }
 }
 
-// MINB blocks per SM: 3 for passes of one wave or less (shortest tile
-// latency), 4 for longer passes (more tiles in flight).  Passes of four blocks
-// and of tiles above the full size load the values late.
+// MINB blocks per SM: 3 (shortest tile latency) or 4 (more tiles in flight), as
+// dispatch_pass says.  Passes of four blocks and of tiles above the full size load
+// the values late.
 template <typename K, int RBITS, int ITEMS, typename W, int MINB, bool ONCE>
 __global__ void __launch_bounds__(kSortBlock, MINB) onesweep_kernel(PassArgs<K> a) {
     using L = PassSmem<K, RBITS, ITEMS>;

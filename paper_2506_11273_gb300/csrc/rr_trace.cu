@@ -1250,8 +1250,9 @@ namespace {
 
 // Launches of at most this many rays put four lanes to a ray (two lanes are
 // better than neither one nor four at any size).  Random order, one against four
-// lanes, us; tiny scene: 4,097 rays 50 / 40, 8,192 52 / 44, 16,384 53 / 51, 30,000
-// 57 / 63; 1,168,576 triangles: 16,384 92 / 83, 38,912 97 / 102.
+// lanes, us; tiny scene: 4,097 rays 48 / 38, 8,192 49 / 40, 16,384 49 / 46, 25,000
+// 53 / 56 (camera rays 16,384 36 / 37); 1,168,576 triangles: 16,384 85 / 74, 38,912
+// 100 / 101.
 constexpr uint32_t kQuadRays = 16384;
 
 template <bool QUAD, bool ACC, bool ANY, bool MULTI, int BLOCK>
